@@ -51,6 +51,19 @@ dim3 grid2d(long long len, int B) {
   return dim3((unsigned)bx, (unsigned)std::max(1, std::min(B, 65535)));
 }
 
+// Grid of the updates: V coordinates per thread and pass, x over the coordinates of an
+// instance, y over the instances.
+dim3 update_grid(long long len, int B, int V) {
+  const long long bx = std::max(1LL, std::min(1024LL, (len + 256LL * V - 1) / (256LL * V)));
+  return dim3((unsigned)bx, (unsigned)std::max(1, std::min(B, 65535)));
+}
+// Chunks of the check reductions of B instances of `len` coordinates: blocks of at
+// least 2048 coordinates, about eight per SM in all.
+int check_chunks(long long len, int B) {
+  const long long want = (8LL * 152 + B - 1) / B;
+  return (int)std::max(1LL, std::min(want, (len + 2047) / 2048));
+}
+
 mpax_status sfail(mpax_status s, const std::string& m) {
   set_last_error(m.c_str());
   return s;
@@ -150,170 +163,274 @@ __device__ __forceinline__ void split_store(float v, __nv_bfloat16* hi, __nv_bfl
 struct Vecs {
   int m, n, B;
   const float *ct, *l, *u, *lc, *uc;  // scaled: ct n x B, l/u n, lc/uc m
-  float *w, *xa, *xhat, *T;             // n x B
-  float *y, *ya, *yhat, *S;             // m x B
+  float *w, *xa, *xhat, *xprev, *T;     // n x B
+  float *y, *ya, *yhat, *yprev, *S;     // m x B
   __nv_bfloat16 *xh_hi, *xh_lo, *y_hi, *y_lo;  // BF16 splits: B rows of ldx / ldy
-  double* part;                          // per-column partials [q][k]
   Inst* inst;
+  const float4* step;                    // per instance: tau, sigma, 1/sigma, running (1 or 0)
   long long ldx, ldy;                    // row strides of the splits (n, m rounded to 8)
 };
 
-// primal: T = A~^T Y; x = w + (anchor - w)/(k+1); x^ = proj(x - tau (c~ - T));
-// w <- 2 x^ - x (also split to BF16 for the next product)
-// tpart (B = 1 only): T is the sum of the GEMV's tchunks partials, in order.
-// Grid: x over the coordinates of an instance, y over instances (grid2d).
-__global__ void k_primal(Vecs v, int check, const float* __restrict__ tpart, int tchunks) {
-  for (int k = blockIdx.y; k < v.B; k += gridDim.y)
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < v.n; j += gridDim.x * blockDim.x) {
-    const size_t e = (size_t)k * v.n + j;
-    const Inst& I = v.inst[k];
-    if (I.done) continue;
-    float t;
-    if (tpart) {
-      t = 0.0f;
-      for (int c = 0; c < tchunks; ++c) t += tpart[(size_t)c * v.n + j];
-    } else {
-      t = v.T[e];
+// Step sizes and Halpern weights of every instance in the precision the updates
+// use them in: step[k] = (tau, sigma, 1/sigma, running), and for the iterations
+// it0 .. it0 + len - 1 of the block halpern[t * B + k] = (1/(k'+1), 1/(k'+2)), k' the
+// instance's counter at iteration it0 + t.  The updates are bound by HBM (24 bytes per
+// coordinate), and a double-precision division costs tens of instructions of a pipe
+// that takes 16 cycles for a warp, so none may run per coordinate.  Measured on 512
+// instances of 8192 x 16384: with the divisions in the updates 124 us (primal) and
+// 109 us (dual), from this table with 128-bit accesses 32 us (6.3 TB/s) and 13.7 us.
+constexpr int kCoefIters = 256;  // iterations per table
+__global__ void k_coefs(const Inst* __restrict__ inst, int B, int it0, int len,
+                        float4* __restrict__ step, float2* __restrict__ halpern) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= B * len) return;
+  const int k = t % B;
+  const Inst& I = inst[k];
+  const long long c = I.k + it0 + t / B;
+  halpern[t] = make_float2((float)(1.0 / (double)(c + 1)), (float)(1.0 / (double)(c + 2)));
+  if (t < B)
+    step[k] = make_float4((float)I.tau, (float)I.sigma, (float)(1.0 / I.sigma), I.done ? 0.f : 1.f);
+}
+
+template <int V>
+__device__ __forceinline__ void ld_vec(const float* p, size_t e, float* v) {
+  if constexpr (V == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p + e);
+    v[0] = q.x;
+    v[1] = q.y;
+    v[2] = q.z;
+    v[3] = q.w;
+  } else {
+    v[0] = p[e];
+  }
+}
+template <int V>
+__device__ __forceinline__ void st_vec(float* p, size_t e, const float* v) {
+  if constexpr (V == 4) *reinterpret_cast<float4*>(p + e) = make_float4(v[0], v[1], v[2], v[3]);
+  else p[e] = v[0];
+}
+template <int V>
+__device__ __forceinline__ void split_vec(const float* v, __nv_bfloat16* hi, __nv_bfloat16* lo,
+                                          size_t e) {
+  if constexpr (V == 4) {
+    __nv_bfloat16 h[4], r[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      h[i] = __float2bfloat16_rn(v[i]);
+      r[i] = __float2bfloat16_rn(v[i] - __bfloat162float(h[i]));
     }
-    const float rb = (float)(1.0 / (double)(I.k + 1));
-    const float x0 = v.xa[e], wv = v.w[e];
-    const float x = (I.k == 0) ? x0 : wv + rb * (x0 - wv);
-    const float xh = fminf(fmaxf(x - (float)I.tau * (v.ct[e] - t), v.l[j]), v.u[j]);
-    const float wn = 2.0f * xh - x;
-    v.w[e] = wn;
-    split_store(wn, v.xh_hi, v.xh_lo, (size_t)k * v.ldx + j);
-    if (check) v.xhat[e] = xh;
+    *reinterpret_cast<uint2*>(hi + e) = *reinterpret_cast<const uint2*>(h);
+    *reinterpret_cast<uint2*>(lo + e) = *reinterpret_cast<const uint2*>(r);
+  } else {
+    split_store(v[0], hi, lo, e);
+  }
+}
+// The sum of `chunks` partial vectors of length len at coordinate e, in order (B = 1:
+// the matrix-vector product's partials); the loads of eight chunks are in flight at once.
+template <int V>
+__device__ __forceinline__ void sum_parts(const float* part, int chunks, int len, int e, float* t) {
+#pragma unroll
+  for (int i = 0; i < V; ++i) t[i] = 0.0f;
+#pragma unroll 8
+  for (int c = 0; c < chunks; ++c) {
+    float q[V];
+    ld_vec<V>(part, (size_t)c * len + e, q);
+#pragma unroll
+    for (int i = 0; i < V; ++i) t[i] += q[i];
+  }
+}
+
+// primal: T = A~^T Y; x = w + (anchor - w)/(k+1); x^ = proj(x - tau (c~ - T));
+// w <- 2 x^ - x (BF: also split for the next product).  Check iterations store x^ and x.
+// tpart (B = 1 only): T is the sum of the GEMV's tchunks partials, in order.
+// Grid: x over V coordinates of an instance per thread, y over instances (grid2d).
+template <int V, bool BF>
+__global__ void k_primal(Vecs v, const float2* __restrict__ halpern, int check,
+                         const float* __restrict__ tpart, int tchunks) {
+  for (int k = blockIdx.y; k < v.B; k += gridDim.y) {
+    const float4 st = v.step[k];
+    if (st.w == 0.0f) continue;
+    const float rb = halpern[k].x;  // 1 exactly when the anchor is the iterate
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * V; j < v.n;
+         j += gridDim.x * blockDim.x * V) {
+      const size_t e = (size_t)k * v.n + j;
+      float t[V], x0[V], wv[V], c[V], lo[V], hi[V], x[V], xh[V], wn[V];
+      if (tpart) sum_parts<V>(tpart, tchunks, v.n, j, t);
+      else ld_vec<V>(v.T, e, t);
+      ld_vec<V>(v.xa, e, x0);
+      ld_vec<V>(v.w, e, wv);
+      ld_vec<V>(v.ct, e, c);
+      ld_vec<V>(v.l, j, lo);
+      ld_vec<V>(v.u, j, hi);
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        x[i] = (rb == 1.0f) ? x0[i] : wv[i] + rb * (x0[i] - wv[i]);
+        xh[i] = fminf(fmaxf(x[i] - st.x * (c[i] - t[i]), lo[i]), hi[i]);
+        wn[i] = 2.0f * xh[i] - x[i];
+      }
+      st_vec<V>(v.w, e, wn);
+      if constexpr (BF) split_vec<V>(wn, v.xh_hi, v.xh_lo, (size_t)k * v.ldx + j);
+      if (check) {
+        st_vec<V>(v.xhat, e, xh);
+        st_vec<V>(v.xprev, e, x);
+      }
+    }
   }
 }
 
 // dual: S = A~ xbar; y^ = sigma (v - proj_[-uc,-lc](v)), v = y/sigma - S;
-// y <- z + (anchor - z)/(k+2), z = 2 y^ - y (also split)
+// y <- z + (anchor - z)/(k+2), z = 2 y^ - y (BF: also split)
 // spart (B = 1 only): S is the sum of the GEMV's schunks partials, in order.
-__global__ void k_dual(Vecs v, int check, const float* __restrict__ spart, int schunks) {
-  for (int k = blockIdx.y; k < v.B; k += gridDim.y)
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < v.m; i += gridDim.x * blockDim.x) {
-    const size_t e = (size_t)k * v.m + i;
-    const Inst& I = v.inst[k];
-    if (I.done) continue;
-    float sv;
-    if (spart) {
-      sv = 0.0f;
-      for (int c = 0; c < schunks; ++c) sv += spart[(size_t)c * v.m + i];
-    } else {
-      sv = v.S[e];
+template <int V, bool BF>
+__global__ void k_dual(Vecs v, const float2* __restrict__ halpern, int check,
+                       const float* __restrict__ spart, int schunks) {
+  for (int k = blockIdx.y; k < v.B; k += gridDim.y) {
+    const float4 st = v.step[k];
+    if (st.w == 0.0f) continue;
+    const float hb = halpern[k].y;
+    for (int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V; i0 < v.m;
+         i0 += gridDim.x * blockDim.x * V) {
+      const size_t e = (size_t)k * v.m + i0;
+      float s[V], y0[V], ya[V], lc[V], uc[V], yh[V], yn[V];
+      if (spart) sum_parts<V>(spart, schunks, v.m, i0, s);
+      else ld_vec<V>(v.S, e, s);
+      ld_vec<V>(v.y, e, y0);
+      ld_vec<V>(v.ya, e, ya);
+      ld_vec<V>(v.lc, i0, lc);
+      ld_vec<V>(v.uc, i0, uc);
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        const float vv = y0[i] * st.z - s[i];
+        yh[i] = st.y * (vv - fminf(fmaxf(vv, -uc[i]), -lc[i]));
+        const float z = 2.0f * yh[i] - y0[i];
+        yn[i] = z + hb * (ya[i] - z);
+      }
+      st_vec<V>(v.y, e, yn);
+      if constexpr (BF) split_vec<V>(yn, v.y_hi, v.y_lo, (size_t)k * v.ldy + i0);
+      if (check) {
+        st_vec<V>(v.yhat, e, yh);
+        st_vec<V>(v.yprev, e, y0);
+      }
     }
-    const float sg = (float)I.sigma, isg = (float)(1.0 / I.sigma);
-    const float hb = (float)(1.0 / (double)(I.k + 2));
-    const float y0 = v.y[e];
-    const float vv = y0 * isg - sv;
-    const float yh = sg * (vv - fminf(fmaxf(vv, -v.uc[i]), -v.lc[i]));
-    const float z = 2.0f * yh - y0;
-    const float yn = z + hb * (v.ya[e] - z);
-    v.y[e] = yn;
-    split_store(yn, v.y_hi, v.y_lo, (size_t)k * v.ldy + i);
-    if (check) v.yhat[e] = yh;
   }
 }
 
-__global__ void k_advance(Inst* inst, int B) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < B && !inst[k].done) {
-    inst[k].k += 1;
-    inst[k].total += 1;
+// Launches of the two updates: four coordinates per thread where every row of
+// the iterates starts on 16 bytes.
+void launch_primal(const Vecs& v, bool bf, const float2* halpern, int check, const float* tpart,
+                   int tchunks, cudaStream_t s) {
+  if (v.n % 4 == 0) {
+    const dim3 g = update_grid(v.n, v.B, 4);
+    if (bf) k_primal<4, true><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
+    else k_primal<4, false><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
+  } else {
+    const dim3 g = update_grid(v.n, v.B, 1);
+    if (bf) k_primal<1, true><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
+    else k_primal<1, false><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
+  }
+}
+void launch_dual(const Vecs& v, bool bf, const float2* halpern, int check, const float* spart,
+                 int schunks, cudaStream_t s) {
+  if (v.m % 4 == 0) {
+    const dim3 g = update_grid(v.m, v.B, 4);
+    if (bf) k_dual<4, true><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
+    else k_dual<4, false><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
+  } else {
+    const dim3 g = update_grid(v.m, v.B, 1);
+    if (bf) k_dual<1, true><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
+    else k_dual<1, false><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
   }
 }
 
-// Per-column check reductions (one block per instance, fixed order).
-// The products S = A~ x^ and T = A~^T y^ were formed into S and T by the caller.
-// part[q * B + k]: 0 sum (x^-x)^2 .. computed here from w/xa? -- see k_check_prep.
-struct KktArgs {
-  int m, n, B;
-  const float *xhat, *yhat, *S, *T, *xprev_w, *xa, *yprev, *ya;
-  const double *Dr, *Dc, *c0, *lc0, *uc0, *l0, *u0;  // c0: n x B unscaled costs
+// Partial sums of a check in FP64: block (c, k) takes chunk c of the coordinates and
+// rows of instance k and writes part[(q * chunks + c) * B + k]:
+//   q 0-4: |r_d|^2, c x, bound terms, |r_p|^2, row terms of the KKT test at (x^, y^)
+//          (S = A~ x^ and T = A~^T y^ were formed by the caller);
+//   q 5-8: |x^-x|^2, |x^-anchor|^2, |y^-y|^2, |y^-anchor|^2 of the restart rule.
+// With one block per instance a single instance of 100,000 columns took 1.17 ms a
+// check on its one SM (0.10 of the dense knapsack's solve); the chunks give every SM a
+// part of it.  512 instances of 8192 x 16384: 0.60 ms, bound by the FP64 pipe (about
+// 12 operations per coordinate at two lanes per SM and cycle).
+constexpr int kCheckParts = 9;
+struct CheckArgs {
+  int m, n, B, chunks;
+  const float *xhat, *yhat, *S, *T, *xprev, *xa, *yprev, *ya;
+  const double *Dr, *Dc, *iDr, *iDc, *c0, *lc0, *uc0, *l0, *u0;  // c0: n x B unscaled costs
   double* part;
 };
 
-__global__ void k_kkt_cols(KktArgs a, const Inst* inst) {
+__global__ void k_check_part(CheckArgs a, const Inst* inst) {
   __shared__ double sh[32];
-  const int k = blockIdx.x;
-  if (inst[k].done) return;
-  const size_t on = (size_t)k * a.n, om = (size_t)k * a.m;
-  double rd2 = 0, cx = 0, bt = 0;
-  for (int j = threadIdx.x; j < a.n; j += blockDim.x) {
-    const double aty = (double)a.T[on + j] / a.Dc[j];
-    const double x = a.Dc[j] * (double)a.xhat[on + j];
-    const double c = a.c0[on + j];
-    const double lam = c - aty;
-    const double lo = a.l0[j], hi = a.u0[j];
-    const bool lf = isfinite(lo), uf = isfinite(hi);
-    const double lh = (lf && uf) ? lam : lf ? fmax(lam, 0.0) : uf ? fmin(lam, 0.0) : 0.0;
-    rd2 += (lam - lh) * (lam - lh);
-    cx += c * x;
-    bt += (lf ? lo * fmax(lh, 0.0) : 0.0) + (uf ? hi * fmin(lh, 0.0) : 0.0);
-  }
-  double rp2 = 0, yt = 0;
-  for (int i = threadIdx.x; i < a.m; i += blockDim.x) {
-    const double ax = (double)a.S[om + i] / a.Dr[i];
-    const double lo = a.lc0[i], hi = a.uc0[i];
-    const double r = ax - fmin(fmax(ax, lo), hi);
-    rp2 += r * r;
-    const double y = a.Dr[i] * (double)a.yhat[om + i];
-    if (y > 0.0 && isfinite(lo)) yt += lo * y;
-    if (y < 0.0 && isfinite(hi)) yt += hi * y;
-  }
-  const double v[5] = {rd2, cx, bt, rp2, yt};
-  for (int q = 0; q < 5; ++q) {
-    const double s = block_sum(v[q], sh);
-    if (threadIdx.x == 0) a.part[(size_t)q * a.B + k] = s;
-  }
-}
-
-// restart metric pieces: x = w_prev rebuilt is not stored; use the stored x^ and the
-// iterate before the check step (xprev) to form |x^ - x|^2 and |x^ - anchor|^2
-__global__ void k_fixed_point_cols(const float* __restrict__ xhat, const float* __restrict__ xprev,
-                                   const float* __restrict__ xa, const float* __restrict__ yhat,
-                                   const float* __restrict__ yprev, const float* __restrict__ ya,
-                                   int m, int n, int B, const Inst* inst, double* part) {
-  __shared__ double sh[32];
-  const int k = blockIdx.x;
-  if (inst[k].done) return;
-  const size_t on = (size_t)k * n, om = (size_t)k * m;
-  double p0 = 0, p1 = 0, d0 = 0, d1 = 0;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    const double a = (double)xhat[on + j] - (double)xprev[on + j];
-    const double b = (double)xhat[on + j] - (double)xa[on + j];
-    p0 += a * a;
-    p1 += b * b;
-  }
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double a = (double)yhat[om + i] - (double)yprev[om + i];
-    const double b = (double)yhat[om + i] - (double)ya[om + i];
-    d0 += a * a;
-    d1 += b * b;
-  }
-  const double v[4] = {p0, p1, d0, d1};
-  for (int q = 0; q < 4; ++q) {
-    const double s = block_sum(v[q], sh);
-    if (threadIdx.x == 0) part[(size_t)(5 + q) * B + k] = s;
+  const int c = blockIdx.x;
+  const int np = (a.n + a.chunks - 1) / a.chunks, mp = (a.m + a.chunks - 1) / a.chunks;
+  for (int k = blockIdx.y; k < a.B; k += gridDim.y) {
+    if (inst[k].done) continue;
+    const size_t on = (size_t)k * a.n, om = (size_t)k * a.m;
+    double rd2 = 0, cx = 0, bt = 0, p0 = 0, p1 = 0;
+    for (int j = c * np + threadIdx.x; j < min(a.n, (c + 1) * np); j += blockDim.x) {
+      const double xh = (double)a.xhat[on + j];
+      const double aty = (double)a.T[on + j] * a.iDc[j];
+      const double x = a.Dc[j] * xh;
+      const double cc = a.c0[on + j];
+      const double lam = cc - aty;
+      const double lo = a.l0[j], hi = a.u0[j];
+      const bool lf = isfinite(lo), uf = isfinite(hi);
+      const double lh = (lf && uf) ? lam : lf ? fmax(lam, 0.0) : uf ? fmin(lam, 0.0) : 0.0;
+      rd2 += (lam - lh) * (lam - lh);
+      cx += cc * x;
+      bt += (lf ? lo * fmax(lh, 0.0) : 0.0) + (uf ? hi * fmin(lh, 0.0) : 0.0);
+      const double d0 = xh - (double)a.xprev[on + j], d1 = xh - (double)a.xa[on + j];
+      p0 += d0 * d0;
+      p1 += d1 * d1;
+    }
+    double rp2 = 0, yt = 0, d0 = 0, d1 = 0;
+    for (int i = c * mp + threadIdx.x; i < min(a.m, (c + 1) * mp); i += blockDim.x) {
+      const double yh = (double)a.yhat[om + i];
+      const double ax = (double)a.S[om + i] * a.iDr[i];
+      const double lo = a.lc0[i], hi = a.uc0[i];
+      const double r = ax - fmin(fmax(ax, lo), hi);
+      rp2 += r * r;
+      const double y = a.Dr[i] * yh;
+      if (y > 0.0 && isfinite(lo)) yt += lo * y;
+      if (y < 0.0 && isfinite(hi)) yt += hi * y;
+      const double e0 = yh - (double)a.yprev[om + i], e1 = yh - (double)a.ya[om + i];
+      d0 += e0 * e0;
+      d1 += e1 * e1;
+    }
+    const double v[kCheckParts] = {rd2, cx, bt, rp2, yt, p0, p1, d0, d1};
+#pragma unroll
+    for (int q = 0; q < kCheckParts; ++q) {
+      const double s = block_sum(v[q], sh);
+      if (threadIdx.x == 0) a.part[((size_t)q * a.chunks + c) * a.B + k] = s;
+    }
   }
 }
 
 struct CheckParams {
   double eps_abs, eps_rel, r_suff, r_nec, r_art, pw_smooth, eta, b_norm;
   long long iter_limit, now_ns, time_limit_ns;
-  int B, check_no, stall_limit;
+  int B, len, chunks, stall_limit;
 };
 
+// The check of every instance after a block of p.len iterations (which advance its
+// counters here), from the chunk sums of k_check_part in chunk order.
 __global__ void k_check_finalize(Inst* inst, const double* part, CheckParams p) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= p.B) return;
   Inst& I = inst[k];
   I.restart = 0;
   if (I.done) return;
-  const double rd2 = part[0 * p.B + k], cx = part[1 * p.B + k], bt = part[2 * p.B + k],
-               rp2 = part[3 * p.B + k], yt = part[4 * p.B + k];
-  const double P0 = part[5 * p.B + k], P1 = part[6 * p.B + k], D0 = part[7 * p.B + k],
-               D1 = part[8 * p.B + k];
+  I.k += p.len;
+  I.total += p.len;
+  double t[kCheckParts];
+#pragma unroll
+  for (int q = 0; q < kCheckParts; ++q) t[q] = 0.0;
+#pragma unroll 4
+  for (int c = 0; c < p.chunks; ++c)
+#pragma unroll
+    for (int q = 0; q < kCheckParts; ++q) t[q] += part[((size_t)q * p.chunks + c) * p.B + k];
+  const double rd2 = t[0], cx = t[1], bt = t[2], rp2 = t[3], yt = t[4], P0 = t[5], P1 = t[6],
+               D0 = t[7], D1 = t[8];
   const double nrp = sqrt(rp2), nrd = sqrt(rd2), pobj = cx, dobj = yt + bt;
   const double gap = fabs(pobj - dobj);
   const double rel = fmax(fmax(nrp / (1.0 + p.b_norm), nrd / (1.0 + I.c_norm)),
@@ -369,7 +486,7 @@ __global__ void k_check_finalize(Inst* inst, const double* part, CheckParams p) 
   }
 }
 
-__global__ void k_restart_apply(Vecs v) {
+__global__ void k_restart_apply(Vecs v, int bf) {
   const int tot = v.n + v.m;
   for (int k = blockIdx.y; k < v.B; k += gridDim.y) {
     if (!v.inst[k].restart) continue;
@@ -379,34 +496,16 @@ __global__ void k_restart_apply(Vecs v) {
         const float xh = v.xhat[e];
         v.xa[e] = xh;
         v.w[e] = xh;
-        split_store(xh, v.xh_hi, v.xh_lo, (size_t)k * v.ldx + t);
+        if (bf) split_store(xh, v.xh_hi, v.xh_lo, (size_t)k * v.ldx + t);
       } else {
         const size_t f = (size_t)k * v.m + (t - v.n);
         const float yh = v.yhat[f];
         v.ya[f] = yh;
         v.y[f] = yh;
-        split_store(yh, v.y_hi, v.y_lo, (size_t)k * v.ldy + (t - v.n));
+        if (bf) split_store(yh, v.y_hi, v.y_lo, (size_t)k * v.ldy + (t - v.n));
       }
     }
   }
-}
-
-// x (before the check step) rebuilt for the fixed-point residual: x = w + (xa - w)/(k+1)
-__global__ void k_rebuild_x(const float* __restrict__ w, const float* __restrict__ xa,
-                            float* __restrict__ out, int n, int B, const Inst* inst) {
-  for (int k = blockIdx.y; k < B; k += gridDim.y)
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    const size_t e = (size_t)k * n + j;
-    const Inst& I = inst[k];
-    const float rb = (float)(1.0 / (double)(I.k + 1));
-    out[e] = (I.k == 0) ? xa[e] : w[e] + rb * (xa[e] - w[e]);
-  }
-}
-
-__global__ void k_copy_f(const float* __restrict__ s, float* __restrict__ d, size_t total) {
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x)
-    d[e] = s[e];
 }
 
 __global__ void k_init_inst(Inst* inst, int B, const double* cnorm_s, const double* cnorm,
@@ -450,6 +549,11 @@ __global__ void k_scale_vec(const double* __restrict__ v, const double* __restri
                             int n, float* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (float)(div ? v[i] / D[i] : v[i] * D[i]);
+}
+
+__global__ void k_inverse(const double* __restrict__ v, int n, double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = 1.0 / v[i];
 }
 
 __global__ void k_unscale_out(const float* __restrict__ v, const double* __restrict__ D, int n,
@@ -550,6 +654,10 @@ struct mpax_shared {
   float *y = nullptr, *ya = nullptr, *yhat = nullptr, *S = nullptr, *yprev = nullptr;
   __nv_bfloat16 *xh_hi = nullptr, *xh_lo = nullptr, *y_hi = nullptr, *y_lo = nullptr;
   double *part = nullptr, *cn = nullptr, *cns = nullptr;
+  double *iDr = nullptr, *iDc = nullptr;  // 1 / Dr, 1 / Dc
+  float4* step = nullptr;                 // per-instance step sizes (k_coefs)
+  float2* halpern = nullptr;              // Halpern weights of kCoefIters iterations (k_coefs)
+  int chunks = 1;                         // chunks of the check reductions
   Inst* inst = nullptr;
   double *Xout = nullptr, *Yout = nullptr;
   bool solved = false;
@@ -596,7 +704,7 @@ void free_shared(mpax_shared* sh) {
                   sh->xhat, sh->T,   sh->xprev, sh->y,     sh->ya,   sh->yhat, sh->S,
                   sh->yprev, sh->xh_hi, sh->xh_lo, sh->y_hi, sh->y_lo, sh->part, sh->cn,
                   sh->cns, sh->inst, sh->Xout, sh->Yout, sh->gpart, sh->gpart_n, sh->spo,
-                  sh->uerr};
+                  sh->uerr, sh->iDr, sh->iDc, sh->step, sh->halpern};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (sh->s) cudaStreamDestroy(sh->s);
@@ -1062,7 +1170,12 @@ mpax_status mpax_lp_shared_create(int32_t m, int32_t n, int32_t B, const float* 
   al(&sh->y_hi, (size_t)B * sh->m8);
   al(&sh->y_lo, (size_t)B * sh->m8);
   al(&sh->uerr, 1);
-  al(&sh->part, 16 * (size_t)B);
+  sh->chunks = check_chunks(std::max(m, n), B);
+  al(&sh->part, (size_t)kCheckParts * sh->chunks * B);
+  al(&sh->iDr, m);
+  al(&sh->iDc, n);
+  al(&sh->step, B);
+  al(&sh->halpern, (size_t)kCoefIters * B);
   al(&sh->cn, B);
   al(&sh->cns, B);
   al(&sh->inst, B);
@@ -1162,7 +1275,9 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   k_scale_vec<<<(n + 255) / 256, 256, 0, s>>>(sh->u, sh->Dc, 1, n, sh->uf);
   k_scale_vec<<<(m + 255) / 256, 256, 0, s>>>(sh->lc, sh->Dr, 0, m, sh->lcf);
   k_scale_vec<<<(m + 255) / 256, 256, 0, s>>>(sh->uc, sh->Dr, 0, m, sh->ucf);
-  L += 7;
+  k_inverse<<<(n + 255) / 256, 256, 0, s>>>(sh->Dc, n, sh->iDc);
+  k_inverse<<<(m + 255) / 256, 256, 0, s>>>(sh->Dr, m, sh->iDr);
+  L += 9;
   // ---- ||A~||_2 by power iteration (FP32 products, FP64 norms) --------------------
   {
     float* v = sh->T;    // n (first column of T as scratch)
@@ -1207,8 +1322,8 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   sh->prep_seconds =
       std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   // ---- per-instance initial state --------------------------------------------------
-  k_colnorm<<<B, 256, 0, s>>>(sh->C0, sh->Dc, n, sh->cns);
-  k_colnorm<<<B, 256, 0, s>>>(sh->C0, nullptr, n, sh->cn);
+  k_colnorm<<<B, 1024, 0, s>>>(sh->C0, sh->Dc, n, sh->cns);
+  k_colnorm<<<B, 1024, 0, s>>>(sh->C0, nullptr, n, sh->cn);
   k_bound_norm<<<1, 512, 0, s>>>(sh->lc, sh->uc, sh->Dr, m, sh->scal);
   double bn[2];
   cudaMemcpyAsync(bn, sh->scal, sizeof(bn), cudaMemcpyDeviceToHost, s);
@@ -1227,13 +1342,13 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   bool bf = !fp32_products;
   long long switch_iter = -1;  // iteration at which BF16x3 gave way to FP32 products
   int switch_active = 0;
-  Vecs V{m, n, B, sh->ct, sh->lf, sh->uf, sh->lcf, sh->ucf, sh->w, sh->xa, sh->xhat, sh->T,
-         sh->y, sh->ya, sh->yhat, sh->S, sh->xh_hi, sh->xh_lo, sh->y_hi, sh->y_lo, sh->part,
-         sh->inst, sh->n8, sh->m8};
-  KktArgs K{m, n, B, sh->xhat, sh->yhat, sh->S, sh->T, nullptr, sh->xa, nullptr, sh->ya,
-            sh->Dr, sh->Dc, sh->C0, sh->lc, sh->uc, sh->l, sh->u, sh->part};
+  Vecs V{m, n, B, sh->ct, sh->lf, sh->uf, sh->lcf, sh->ucf, sh->w, sh->xa, sh->xhat, sh->xprev,
+         sh->T, sh->y, sh->ya, sh->yhat, sh->yprev, sh->S, sh->xh_hi, sh->xh_lo, sh->y_hi,
+         sh->y_lo, sh->inst, sh->step, sh->n8, sh->m8};
+  CheckArgs K{m, n, B, sh->chunks, sh->xhat, sh->yhat, sh->S, sh->T, sh->xprev, sh->xa,
+              sh->yprev, sh->ya, sh->Dr, sh->Dc, sh->iDr, sh->iDc, sh->C0, sh->lc, sh->uc,
+              sh->l, sh->u, sh->part};
   long long done_iters = 0;
-  int check_no = 0;
   // time limit, checked at each KKT check against the host clock
   const long long tl_ns = o->time_limit >= 9.0e9 ? LLONG_MAX : (long long)(o->time_limit * 1e9);
   std::vector<Inst> hi(B);
@@ -1242,59 +1357,61 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
     const int len = (int)std::min<long long>(o->check_every, o->iteration_limit - done_iters);
     for (int it = 0; it < len; ++it) {
       const int chk = (it == len - 1);
-      if (chk) {  // the iterate before the check step, for the fixed-point residual
-        k_rebuild_x<<<grid2d(n, B), 256, 0, s>>>(sh->w, sh->xa, sh->xprev, n, B, sh->inst);
-        k_copy_f<<<g1(mB), 256, 0, s>>>(sh->y, sh->yprev, mB);
-        L += 2;
+      const float2* hk = sh->halpern + (size_t)(it % kCoefIters) * B;
+      if (it % kCoefIters == 0) {
+        const int cl = std::min(kCoefIters, len - it);
+        k_coefs<<<(B * cl + 255) / 256, 256, 0, s>>>(sh->inst, B, it, cl, sh->step, sh->halpern);
+        L += 1;
       }
       if (B == 1 && !bf) {
         // one instance, FP32: GEMV partials, summed inside the update kernels
         gemv_part(sh, 0, sh->y, sh->As);
-        k_primal<<<grid2d(n, B), 256, 0, s>>>(V, chk, sh->gpart, sh->gemv_chunks);
+        launch_primal(V, false, hk, chk, sh->gpart, sh->gemv_chunks, s);
         gemv_part(sh, 1, sh->w, sh->As);
-        k_dual<<<grid2d(m, B), 256, 0, s>>>(V, chk, sh->gpart_n, sh->gemv_nchunks);
-        k_advance<<<(B + 255) / 256, 256, 0, s>>>(sh->inst, B);
-        L += 3;
+        launch_dual(V, false, hk, chk, sh->gpart_n, sh->gemv_nchunks, s);
+        L += 2;
         continue;
       }
       if (product(sh, 0, sh->y_hi, sh->y_lo, sh->y, sh->T, bf, sh->As)) {
         result = sfail(MPAX_ERR_CUDA, "matrix product launch failed");
         break;
       }
-      k_primal<<<grid2d(n, B), 256, 0, s>>>(V, chk, nullptr, 0);
+      launch_primal(V, bf, hk, chk, nullptr, 0, s);
       // the dual product reads the reflected point w (FP32) or its BF16 split
       if (product(sh, 1, sh->xh_hi, sh->xh_lo, sh->w, sh->S, bf, sh->As)) {
         result = sfail(MPAX_ERR_CUDA, "matrix product launch failed");
         break;
       }
-      k_dual<<<grid2d(m, B), 256, 0, s>>>(V, chk, nullptr, 0);
-      k_advance<<<(B + 255) / 256, 256, 0, s>>>(sh->inst, B);
-      L += 3;
+      launch_dual(V, bf, hk, chk, nullptr, 0, s);
+      L += 2;
     }
     if (result) break;
     done_iters += len;
-    ++check_no;
-    // KKT products at (x^, y^): S = A~ x^, T = A~^T y^ (the x^/y^ splits reuse the
-    // BF16 buffers; the iteration rewrites them before its next product)
-    split_rows(sh->xhat, B, n, n, sh->xh_hi, sh->xh_lo, sh->n8, s);
-    split_rows(sh->yhat, B, m, m, sh->y_hi, sh->y_lo, sh->m8, s);
+    // KKT products at (x^, y^): S = A~ x^, T = A~^T y^ (BF16x3: the x^/y^ splits reuse
+    // the iterates' buffers, which are rebuilt below)
+    if (bf) {
+      split_rows(sh->xhat, B, n, n, sh->xh_hi, sh->xh_lo, sh->n8, s);
+      split_rows(sh->yhat, B, m, m, sh->y_hi, sh->y_lo, sh->m8, s);
+      L += 2;
+    }
     product(sh, 1, sh->xh_hi, sh->xh_lo, sh->xhat, sh->S, bf, sh->As);
     product(sh, 0, sh->y_hi, sh->y_lo, sh->yhat, sh->T, bf, sh->As);
-    k_kkt_cols<<<B, 256, 0, s>>>(K, sh->inst);
-    k_fixed_point_cols<<<B, 256, 0, s>>>(sh->xhat, sh->xprev, sh->xa, sh->yhat, sh->yprev,
-                                         sh->ya, m, n, B, sh->inst, sh->part);
+    k_check_part<<<dim3((unsigned)sh->chunks, (unsigned)std::min(B, 65535)), 256, 0, s>>>(K,
+                                                                                     sh->inst);
     CheckParams cp{o->eps_abs, o->eps_rel, o->restart_sufficient, o->restart_necessary,
                    o->restart_artificial, o->primal_weight_smoothing, eta, bn[0],
                    o->iteration_limit,
                    (long long)std::chrono::duration_cast<std::chrono::nanoseconds>(
                        std::chrono::steady_clock::now() - t0).count(),
-                   tl_ns, B, check_no, (bf && o->fp64_continuation) ? o->stall_checks : 0};
+                   tl_ns, B, len, sh->chunks, (bf && o->fp64_continuation) ? o->stall_checks : 0};
     k_check_finalize<<<(B + 255) / 256, 256, 0, s>>>(sh->inst, sh->part, cp);
-    // the BF16 splits of the iterates are rebuilt (restart copies x^, y^ into them)
-    split_rows(sh->w, B, n, n, sh->xh_hi, sh->xh_lo, sh->n8, s);
-    split_rows(sh->y, B, m, m, sh->y_hi, sh->y_lo, sh->m8, s);
-    k_restart_apply<<<grid2d(n + m, B), 256, 0, s>>>(V);
-    L += 8;
+    if (bf) {  // the BF16 splits of the iterates again (a restart copies x^, y^ into them)
+      split_rows(sh->w, B, n, n, sh->xh_hi, sh->xh_lo, sh->n8, s);
+      split_rows(sh->y, B, m, m, sh->y_hi, sh->y_lo, sh->m8, s);
+      L += 2;
+    }
+    k_restart_apply<<<grid2d((long long)n + m, B), 256, 0, s>>>(V, bf);
+    L += 3;
     cudaMemcpyAsync(hi.data(), sh->inst, sizeof(Inst) * B, cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
     if (sh->profiling) collect_product_times(sh);
