@@ -76,120 +76,11 @@ struct Inst {
   int done, status, restart, have_anchor, stalled;
 };
 
-// ---- dense scaling (row-major m x n): row/column infinity- and 1-norms ----------
-__global__ void k_row_red(const float* __restrict__ A, int m, int n, int sum,
-                          double* __restrict__ out) {
-  __shared__ double sh[32];
-  for (int i = blockIdx.x; i < m; i += gridDim.x) {
-    double acc = 0.0;
-    const float* r = A + (size_t)i * n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      const double v = fabs((double)r[j]);
-      acc = sum ? acc + v : fmax(acc, v);
-    }
-    if (sum) {
-      acc = block_sum(acc, sh);
-    } else {
-      // fixed-order max tree
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc = fmax(acc, __shfl_xor_sync(0xffffffffu, acc, o));
-      __syncthreads();
-      if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-      __syncthreads();
-      if (threadIdx.x < 32) {
-        acc = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc = fmax(acc, __shfl_xor_sync(0xffffffffu, acc, o));
-      }
-    }
-    if (threadIdx.x == 0) out[i] = acc;
-    __syncthreads();
-  }
-}
-
-// column reduction: thread per column, sequential over rows (coalesced in j)
-__global__ void k_col_red(const float* __restrict__ A, int m, int n, int sum,
-                          double* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  double acc = 0.0;
-  for (int i = 0; i < m; ++i) {
-    const double v = fabs((double)A[(size_t)i * n + j]);
-    acc = sum ? acc + v : fmax(acc, v);
-  }
-  out[j] = acc;
-}
-
-__global__ void k_factor(double* __restrict__ norm, int k, double* __restrict__ D) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= k) return;
-  const double v = norm[i];
-  const double d = v > 0.0 ? 1.0 / sqrt(v) : 1.0;
-  norm[i] = d;
-  D[i] *= d;
-}
-
-// dst_ij = (src_ij * dr_i) * dc_j
-__global__ void k_scale_dense(const float* __restrict__ src, float* __restrict__ dst, int m,
-                              int n, const double* __restrict__ dr,
-                              const double* __restrict__ dc) {
-  const size_t total = (size_t)m * n;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / n), j = (int)(e % n);
-    dst[e] = (float)(((double)src[e] * dr[i]) * dc[j]);
-  }
-}
-
-__global__ void k_split(const float* __restrict__ a, __nv_bfloat16* __restrict__ hi,
-                        __nv_bfloat16* __restrict__ lo, size_t total) {
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const float v = a[e];
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    hi[e] = h;
-    lo[e] = __float2bfloat16_rn(v - __bfloat162float(h));
-  }
-}
-
 __device__ __forceinline__ void split_store(float v, __nv_bfloat16* hi, __nv_bfloat16* lo,
                                             size_t e) {
   const __nv_bfloat16 h = __float2bfloat16_rn(v);
   hi[e] = h;
   lo[e] = __float2bfloat16_rn(v - __bfloat162float(h));
-}
-
-// ---- fused updates ----------------------------------------------------------------
-struct Vecs {
-  int m, n, B;
-  const float *ct, *l, *u, *lc, *uc;  // scaled: ct n x B, l/u n, lc/uc m
-  float *w, *xa, *xhat, *xprev, *T;     // n x B
-  float *y, *ya, *yhat, *yprev, *S;     // m x B
-  __nv_bfloat16 *xh_hi, *xh_lo, *y_hi, *y_lo;  // BF16 splits: B rows of ldx / ldy
-  Inst* inst;
-  const float4* step;                    // per instance: tau, sigma, 1/sigma, running (1 or 0)
-  long long ldx, ldy;                    // row strides of the splits (n, m rounded to 8)
-};
-
-// Step sizes and Halpern weights of every instance in the precision the updates
-// use them in: step[k] = (tau, sigma, 1/sigma, running), and for the iterations
-// it0 .. it0 + len - 1 of the block halpern[t * B + k] = (1/(k'+1), 1/(k'+2)), k' the
-// instance's counter at iteration it0 + t.  The updates are bound by HBM (24 bytes per
-// coordinate), and a double-precision division costs tens of instructions of a pipe
-// that takes 16 cycles for a warp, so none may run per coordinate.  Measured on 512
-// instances of 8192 x 16384: with the divisions in the updates 124 us (primal) and
-// 109 us (dual), from this table with 128-bit accesses 32 us (6.3 TB/s) and 13.7 us.
-constexpr int kCoefIters = 256;  // iterations per table
-__global__ void k_coefs(const Inst* __restrict__ inst, int B, int it0, int len,
-                        float4* __restrict__ step, float2* __restrict__ halpern) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= B * len) return;
-  const int k = t % B;
-  const Inst& I = inst[k];
-  const long long c = I.k + it0 + t / B;
-  halpern[t] = make_float2((float)(1.0 / (double)(c + 1)), (float)(1.0 / (double)(c + 2)));
-  if (t < B)
-    step[k] = make_float4((float)I.tau, (float)I.sigma, (float)(1.0 / I.sigma), I.done ? 0.f : 1.f);
 }
 
 template <int V>
@@ -225,6 +116,245 @@ __device__ __forceinline__ void split_vec(const float* v, __nv_bfloat16* hi, __n
     split_store(v[0], hi, lo, e);
   }
 }
+// ---- dense scaling (row-major m x n): Ruiz and Pock-Chambolle rounds -------------
+// One pass over A per Ruiz round: it applies the last round's factors, writes the
+// rescaled value and reduces its row and column maximum.  A tile is kDenseRows rows by
+// 256 V columns; a thread keeps its V column maxima in registers down the tile, a row's
+// V values are reduced across the warp.  Maxima are exact in any order and go through
+// integer atomics on the bit patterns of the non-negative floats.
+//
+// The pass is bound by HBM (one read, and one write from the second round on) only if
+// it keeps off the FP64 pipe (two lanes per SM and cycle), so the scaled value
+// fl32((a r) c), r and c in FP64, is formed from float pairs: r = rh + rl, c = ch + cl
+// to 48 bits and error-free FP32 products give a r c to within 2^-44.  Where that
+// margin leaves the rounding to a float open (about one value in 10^6), or a product
+// leaves the range in which the pairs are exact, the value is formed in FP64: the
+// result is that of the FP64 products, bit for bit (the BF16 splits of the products
+// that follow turn any other last bit into a 2^-17 one).
+// Measured on 8192 x 16384 (0.54 GB): row maxima 0.79 ms, column maxima 1.88 ms and
+// scaling 1.00 ms before; one pass 0.16 ms (6.5 TB/s) now.
+constexpr int kDenseRows = 64;  // rows of a tile
+struct DensePass {
+  const float* src;
+  float* dst;
+  int m, n;
+  int ctiles;                   // column tiles; block b takes tile (b / ctiles, b % ctiles)
+  const float2 *fr, *fc;        // factors as float pairs
+  const double *dr, *dc;        // the same in FP64
+  unsigned *rowmax, *colmax;    // norms of a Ruiz round (float bits, start at 0)
+  __nv_bfloat16 *hi, *lo;       // BF16 split of the result (rows of ldh)
+  long long ldh;
+};
+
+__device__ __forceinline__ float scale_pair(float a, float2 r, float2 c, const double* dr,
+                                            const double* dc) {
+  const float p = a * r.x;
+  const float pl = fmaf(a, r.y, fmaf(a, r.x, -p));
+  const float q = p * c.x;
+  const float ql = fmaf(p, c.y, fmaf(pl, c.x, fmaf(p, c.x, -q)));
+  const float ap = fabsf(p), aq = fabsf(q);
+  const float d = aq * 1.1368684e-13f;  // 2^-43
+  const float up = q + (ql + d), dn = q + (ql - d);
+  // (false for NaN, infinities, zeros and values near the ends of the range)
+  if (up == dn && ap > 1e-22f && ap < 1e30f && aq > 1e-22f && aq < 1e30f) return up;
+  if (a == 0.0f) return a;
+  return (float)(((double)a * *dr) * *dc);
+}
+
+template <int V, bool kFactor, bool kMax, bool kWrite, bool kSplit>
+__global__ void __launch_bounds__(256) k_dense_pass(DensePass a) {
+  __shared__ unsigned srow[kDenseRows];
+  const int ct = blockIdx.x % a.ctiles, rt = blockIdx.x / a.ctiles;
+  const int j = (ct * 256 + threadIdx.x) * V;
+  const int r0 = rt * kDenseRows, r1 = min(a.m, r0 + kDenseRows);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool in = j < a.n;  // V = 4: n is a multiple of 4
+  if (kMax && threadIdx.x < kDenseRows) srow[threadIdx.x] = 0u;
+  if (kMax) __syncthreads();
+  float2 fc[V];
+  float cmax[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) {
+    fc[i] = (kFactor && in) ? a.fc[j + i] : make_float2(1.0f, 0.0f);
+    cmax[i] = 0.0f;
+  }
+  constexpr int U = 4;  // rows in flight
+  for (int rb = r0; rb < r1; rb += U) {
+    float v[U][V];
+#pragma unroll
+    for (int t = 0; t < U; ++t) {
+#pragma unroll
+      for (int i = 0; i < V; ++i) v[t][i] = 0.0f;
+      if (in && rb + t < r1) ld_vec<V>(a.src, (size_t)(rb + t) * a.n + j, v[t]);
+    }
+#pragma unroll
+    for (int t = 0; t < U; ++t) {
+      const int r = rb + t;
+      if (r >= r1) break;
+      if constexpr (kFactor) {
+        const float2 fr = a.fr[r];
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+          if (in) v[t][i] = scale_pair(v[t][i], fr, fc[i], a.dr + r, a.dc + j + i);
+      }
+      if (kWrite && in) st_vec<V>(a.dst, (size_t)r * a.n + j, v[t]);
+      if constexpr (kSplit) {
+        if (in) split_vec<V>(v[t], a.hi, a.lo, (size_t)r * a.ldh + j);
+      }
+      if constexpr (kMax) {
+        float rm = 0.0f;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+          const float w = fabsf(v[t][i]);
+          rm = fmaxf(rm, w);
+          cmax[i] = fmaxf(cmax[i], w);
+        }
+        const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(rm));
+        if (lane == 0) atomicMax(&srow[r - r0], wm);
+      }
+    }
+  }
+  if constexpr (kMax) {
+#pragma unroll
+    for (int i = 0; i < V; ++i)
+      if (in) atomicMax(a.colmax + j + i, __float_as_uint(cmax[i]));
+    __syncthreads();
+    if (threadIdx.x < r1 - r0) atomicMax(a.rowmax + r0 + threadIdx.x, srow[threadIdx.x]);
+  }
+}
+
+// Pock-Chambolle norms in FP64: row sums, a block per row (each thread every 256th
+// value, then a fixed tree), and column sums, a thread per column down the rows in
+// blocks of kColThreads.  The column sums are bound by the FP64 pipe of the SMs that
+// hold a block (a conversion and an addition per value), hence blocks narrower than
+// 256, and by the loads in flight, hence 32 unconditional ones per thread: 0.75 ms on
+// 8192 x 16384 (1.88 ms with 256 threads and one row at a time; one-warp blocks would
+// reach every SM but read 128 bytes a row, 3.7 ms).  The row sums take 0.53 ms, their
+// FP64 pipe time.
+constexpr int kColThreads = 128;
+__global__ void k_row_sum(const float* __restrict__ A, int m, int n, double* __restrict__ out) {
+  __shared__ double sh[32];
+  for (int i = blockIdx.x; i < m; i += gridDim.x) {
+    double acc = 0.0;
+    const float* r = A + (size_t)i * n;
+#pragma unroll 4
+    for (int j = threadIdx.x; j < n; j += blockDim.x) acc += fabs((double)r[j]);
+    acc = block_sum(acc, sh);
+    if (threadIdx.x == 0) out[i] = acc;
+    __syncthreads();
+  }
+}
+__global__ void __launch_bounds__(kColThreads) k_col_sum(const float* __restrict__ A, int m,
+                                                         int n, double* __restrict__ out) {
+  constexpr int U = 32;
+  const int j = blockIdx.x * kColThreads + threadIdx.x;
+  if (j >= n) return;
+  double acc = 0.0;
+  const float* p = A + j;
+  int i = 0;
+  for (; i + U <= m; i += U, p += (size_t)U * n) {
+    float v[U];
+#pragma unroll
+    for (int t = 0; t < U; ++t) v[t] = p[(size_t)t * n];
+#pragma unroll
+    for (int t = 0; t < U; ++t) acc += fabs((double)v[t]);
+  }
+  for (; i < m; ++i, p += n) acc += fabs((double)*p);
+  out[j] = acc;
+}
+
+__device__ __forceinline__ float2 float_pair(double d) {
+  const float h = (float)d;
+  return make_float2(h, isfinite(h) ? (float)(d - (double)h) : 0.0f);
+}
+
+// The factors of a finished round, d = 1/sqrt(norm) (1 for an empty row or column),
+// rows then columns: D *= d; d (over dr, dc) and its float pair are stored.  Norms are
+// the float bits nmax (reset to zero for the next round) or, without them, dr and dc.
+__global__ void k_dense_factor(int m, int n, unsigned* __restrict__ nmax, double* __restrict__ Dr,
+                               double* __restrict__ Dc, double* __restrict__ dr,
+                               double* __restrict__ dc, float2* __restrict__ fr,
+                               float2* __restrict__ fc) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= m + n) return;
+  const bool row = t < m;
+  const int i = row ? t : t - m;
+  const double v = nmax ? (double)__uint_as_float(nmax[t]) : (row ? dr : dc)[i];
+  if (nmax) nmax[t] = 0u;
+  const double d = v > 0.0 ? 1.0 / sqrt(v) : 1.0;
+  (row ? Dr : Dc)[i] *= d;
+  (row ? dr : dc)[i] = d;
+  (row ? fr : fc)[i] = float_pair(d);
+}
+
+// The accumulated factors (rows then columns): float pairs and inverses.
+__global__ void k_dense_final(int m, int n, const double* __restrict__ Dr,
+                              const double* __restrict__ Dc, float2* __restrict__ fr,
+                              float2* __restrict__ fc, double* __restrict__ iDr,
+                              double* __restrict__ iDc) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= m + n) return;
+  const bool row = t < m;
+  const int i = row ? t : t - m;
+  const double d = (row ? Dr : Dc)[i];
+  (row ? fr : fc)[i] = float_pair(d);
+  (row ? iDr : iDc)[i] = 1.0 / d;
+}
+
+// D = 1, maxima = 0 at the start of a scaling
+__global__ void k_dense_init(int m, int n, double* __restrict__ Dr, double* __restrict__ Dc,
+                             unsigned* __restrict__ nmax) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= m + n) return;
+  if (t < m) Dr[t] = 1.0;
+  else Dc[t - m] = 1.0;
+  nmax[t] = 0u;
+}
+
+// Four columns per thread where every row starts on 16 bytes (the buffers are the
+// library's own), else one.
+int dense_col_tiles(int n) { return (int)(n % 4 == 0 ? (n + 1023LL) / 1024 : (n + 255LL) / 256); }
+
+template <bool kFactor, bool kMax, bool kWrite, bool kSplit>
+void dense_pass(const DensePass& a, cudaStream_t s) {
+  const unsigned g = (unsigned)a.ctiles * (unsigned)((a.m + kDenseRows - 1) / kDenseRows);
+  if (a.n % 4 == 0) k_dense_pass<4, kFactor, kMax, kWrite, kSplit><<<g, 256, 0, s>>>(a);
+  else k_dense_pass<1, kFactor, kMax, kWrite, kSplit><<<g, 256, 0, s>>>(a);
+}
+
+// ---- fused updates ----------------------------------------------------------------
+struct Vecs {
+  int m, n, B;
+  const float *ct, *l, *u, *lc, *uc;  // scaled: ct n x B, l/u n, lc/uc m
+  float *w, *xa, *xhat, *xprev, *T;     // n x B
+  float *y, *ya, *yhat, *yprev, *S;     // m x B
+  __nv_bfloat16 *xh_hi, *xh_lo, *y_hi, *y_lo;  // BF16 splits: B rows of ldx / ldy
+  Inst* inst;
+  const float4* step;                    // per instance: tau, sigma, 1/sigma, running (1 or 0)
+  long long ldx, ldy;                    // row strides of the splits (n, m rounded to 8)
+};
+
+// Step sizes and Halpern weights of every instance in the precision the updates
+// use them in: step[k] = (tau, sigma, 1/sigma, running), and for the iterations
+// it0 .. it0 + len - 1 of the block halpern[t * B + k] = (1/(k'+1), 1/(k'+2)), k' the
+// instance's counter at iteration it0 + t.  The updates are bound by HBM (24 bytes per
+// coordinate), and a double-precision division costs tens of instructions of a pipe
+// that takes 16 cycles for a warp, so none may run per coordinate.  Measured on 512
+// instances of 8192 x 16384: with the divisions in the updates 124 us (primal) and
+// 109 us (dual), from this table with 128-bit accesses 32 us (6.3 TB/s) and 13.7 us.
+constexpr int kCoefIters = 256;  // iterations per table
+__global__ void k_coefs(const Inst* __restrict__ inst, int B, int it0, int len,
+                        float4* __restrict__ step, float2* __restrict__ halpern) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= B * len) return;
+  const int k = t % B;
+  const Inst& I = inst[k];
+  const long long c = I.k + it0 + t / B;
+  halpern[t] = make_float2((float)(1.0 / (double)(c + 1)), (float)(1.0 / (double)(c + 2)));
+  if (t < B)
+    step[k] = make_float4((float)I.tau, (float)I.sigma, (float)(1.0 / I.sigma), I.done ? 0.f : 1.f);
+}
+
 // The sum of `chunks` partial vectors of length len at coordinate e, in order (B = 1:
 // the matrix-vector product's partials); the loads of eight chunks are in flight at once.
 template <int V>
@@ -551,11 +681,6 @@ __global__ void k_scale_vec(const double* __restrict__ v, const double* __restri
   if (i < n) out[i] = (float)(div ? v[i] / D[i] : v[i] * D[i]);
 }
 
-__global__ void k_inverse(const double* __restrict__ v, int n, double* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = 1.0 / v[i];
-}
-
 __global__ void k_unscale_out(const float* __restrict__ v, const double* __restrict__ D, int n,
                               size_t total, double* __restrict__ out) {
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -655,6 +780,9 @@ struct mpax_shared {
   __nv_bfloat16 *xh_hi = nullptr, *xh_lo = nullptr, *y_hi = nullptr, *y_lo = nullptr;
   double *part = nullptr, *cn = nullptr, *cns = nullptr;
   double *iDr = nullptr, *iDc = nullptr;  // 1 / Dr, 1 / Dc
+  float2 *fr = nullptr, *fc = nullptr;    // scaling factors of a pass as float pairs
+  unsigned* nmax = nullptr;               // row then column maxima of a Ruiz round
+  int ctiles = 1;                         // column tiles of a scaling pass
   float4* step = nullptr;                 // per-instance step sizes (k_coefs)
   float2* halpern = nullptr;              // Halpern weights of kCoefIters iterations (k_coefs)
   int chunks = 1;                         // chunks of the check reductions
@@ -704,7 +832,8 @@ void free_shared(mpax_shared* sh) {
                   sh->xhat, sh->T,   sh->xprev, sh->y,     sh->ya,   sh->yhat, sh->S,
                   sh->yprev, sh->xh_hi, sh->xh_lo, sh->y_hi, sh->y_lo, sh->part, sh->cn,
                   sh->cns, sh->inst, sh->Xout, sh->Yout, sh->gpart, sh->gpart_n, sh->spo,
-                  sh->uerr, sh->iDr, sh->iDc, sh->step, sh->halpern};
+                  sh->uerr, sh->iDr, sh->iDc, sh->step, sh->halpern, sh->fr, sh->fc,
+                  sh->nmax};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (sh->s) cudaStreamDestroy(sh->s);
@@ -1174,6 +1303,10 @@ mpax_status mpax_lp_shared_create(int32_t m, int32_t n, int32_t B, const float* 
   al(&sh->part, (size_t)kCheckParts * sh->chunks * B);
   al(&sh->iDr, m);
   al(&sh->iDc, n);
+  sh->ctiles = dense_col_tiles(n);
+  al(&sh->fr, m);
+  al(&sh->fc, n);
+  al(&sh->nmax, (size_t)m + n);
   al(&sh->step, B);
   al(&sh->halpern, (size_t)kCoefIters * B);
   al(&sh->cn, B);
@@ -1199,6 +1332,9 @@ mpax_status mpax_lp_shared_create(int32_t m, int32_t n, int32_t B, const float* 
     if (!e) e = cudaMemset(q, 0, sizeof(__nv_bfloat16) * (size_t)B * sh->n8);
   for (void* q : {(void*)sh->y_hi, (void*)sh->y_lo})
     if (!e) e = cudaMemset(q, 0, sizeof(__nv_bfloat16) * (size_t)B * sh->m8);
+  if (sh->n8 != n)  // the pad columns of the split matrix stay zero
+    for (void* q : {(void*)sh->Ahi, (void*)sh->Alo})
+      if (!e) e = cudaMemset(q, 0, sizeof(__nv_bfloat16) * (size_t)m * sh->n8);
   if (!e) e = cudaMemset(sh->uerr, 0, sizeof(int));
   if (!e) e = cudaMemcpy(sh->A0, A, sizeof(float) * mn, k);
   if (!e) e = cudaMemcpy(sh->C0, C, sizeof(double) * nB, k);
@@ -1223,7 +1359,7 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
     return sfail(MPAX_ERR_INVALID_ARGUMENT, "invalid options (reflection_gamma must be 1)");
   const auto t0 = std::chrono::steady_clock::now();
   const int m = sh->m, n = sh->n, B = sh->B;
-  const size_t mn = (size_t)m * n, nB = (size_t)n * B, mB = (size_t)m * B;
+  const size_t nB = (size_t)n * B, mB = (size_t)m * B;
   cudaStream_t s = sh->s;
   cudaEvent_t ev;
   cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
@@ -1237,31 +1373,37 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   sh->gemm_flops = 0.0;
   sh->gemv_launches = 0;
   // ---- scaling of the shared matrix (Ruiz, Pock-Chambolle) ----------------------
-  auto fill1 = [&](double* p, int cnt) {
-    std::vector<double> ones(cnt, 1.0);
-    cudaMemcpyAsync(p, ones.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice, s);
-    cudaStreamSynchronize(s);
-  };
-  fill1(sh->Dr, m);
-  fill1(sh->Dc, n);
-  cudaMemcpyAsync(sh->As, sh->A0, sizeof(float) * mn, cudaMemcpyDeviceToDevice, s);
+  const int gf = (int)(((long long)m + n + 255) / 256);
+  DensePass D{sh->A0, sh->As, m, n, sh->ctiles, sh->fr, sh->fc, sh->red_m, sh->red_n, sh->nmax,
+              sh->nmax + m, sh->Ahi, sh->Alo, sh->n8};
+  k_dense_init<<<gf, 256, 0, s>>>(m, n, sh->Dr, sh->Dc, sh->nmax);
   for (int t = 0; t < o->ruiz_iters; ++t) {
-    k_row_red<<<std::min(m, 4096), 256, 0, s>>>(sh->As, m, n, 0, sh->red_m);
-    k_col_red<<<(n + 255) / 256, 256, 0, s>>>(sh->As, m, n, 0, sh->red_n);
-    k_factor<<<(m + 255) / 256, 256, 0, s>>>(sh->red_m, m, sh->Dr);
-    k_factor<<<(n + 255) / 256, 256, 0, s>>>(sh->red_n, n, sh->Dc);
-    k_scale_dense<<<g1(mn), 256, 0, s>>>(sh->As, sh->As, m, n, sh->red_m, sh->red_n);
-    L += 5;
+    if (t == 0) dense_pass<false, true, false, false>(D, s);
+    else dense_pass<true, true, true, false>(D, s);
+    if (t > 0) D.src = sh->As;
+    k_dense_factor<<<gf, 256, 0, s>>>(m, n, sh->nmax, sh->Dr, sh->Dc, sh->red_m, sh->red_n,
+                                      sh->fr, sh->fc);
+    L += 2;
   }
   if (o->pock_chambolle) {
-    k_row_red<<<std::min(m, 4096), 256, 0, s>>>(sh->As, m, n, 1, sh->red_m);
-    k_col_red<<<(n + 255) / 256, 256, 0, s>>>(sh->As, m, n, 1, sh->red_n);
-    k_factor<<<(m + 255) / 256, 256, 0, s>>>(sh->red_m, m, sh->Dr);
-    k_factor<<<(n + 255) / 256, 256, 0, s>>>(sh->red_n, n, sh->Dc);
-    L += 4;
+    if (o->ruiz_iters > 0) {
+      dense_pass<true, false, true, false>(D, s);
+      D.src = sh->As;
+      L += 1;
+    }
+    k_row_sum<<<std::min(m, 4096), 256, 0, s>>>(D.src, m, n, sh->red_m);
+    k_col_sum<<<(n + kColThreads - 1) / kColThreads, kColThreads, 0, s>>>(D.src, m, n, sh->red_n);
+    k_dense_factor<<<gf, 256, 0, s>>>(m, n, nullptr, sh->Dr, sh->Dc, sh->red_m, sh->red_n, sh->fr,
+                                      sh->fc);
+    L += 3;
   }
-  k_scale_dense<<<g1(mn), 256, 0, s>>>(sh->A0, sh->As, m, n, sh->Dr, sh->Dc);
-  split_rows(sh->As, m, n, n, sh->Ahi, sh->Alo, sh->n8, s);
+  // the scaled matrix from the original values, with its split when the products use it
+  k_dense_final<<<gf, 256, 0, s>>>(m, n, sh->Dr, sh->Dc, sh->fr, sh->fc, sh->iDr, sh->iDc);
+  D.src = sh->A0;
+  D.dr = sh->Dr;
+  D.dc = sh->Dc;
+  if (fp32_products) dense_pass<true, false, true, false>(D, s);
+  else dense_pass<true, false, true, true>(D, s);
   {
     cudaError_t pe = plan_products(sh, !fp32_products);
     if (pe) {
@@ -1275,9 +1417,7 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   k_scale_vec<<<(n + 255) / 256, 256, 0, s>>>(sh->u, sh->Dc, 1, n, sh->uf);
   k_scale_vec<<<(m + 255) / 256, 256, 0, s>>>(sh->lc, sh->Dr, 0, m, sh->lcf);
   k_scale_vec<<<(m + 255) / 256, 256, 0, s>>>(sh->uc, sh->Dr, 0, m, sh->ucf);
-  k_inverse<<<(n + 255) / 256, 256, 0, s>>>(sh->Dc, n, sh->iDc);
-  k_inverse<<<(m + 255) / 256, 256, 0, s>>>(sh->Dr, m, sh->iDr);
-  L += 9;
+  L += 8;
   // ---- ||A~||_2 by power iteration (FP32 products, FP64 norms) --------------------
   {
     float* v = sh->T;    // n (first column of T as scratch)

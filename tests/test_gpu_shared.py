@@ -240,3 +240,33 @@ def test_shared_iterates_match_oracle(C, iterate_case, fp32, tol):
     for k, r in ref.items():
         assert rel_inf(X[k], r.x) <= tol, (k, rel_inf(X[k], r.x))
         assert rel_inf(Y[k], r.y) <= tol, (k, rel_inf(Y[k], r.y))
+
+
+# The scaling rounds run over tiles of 64 rows by 256 columns (n % 4 != 0) or 1024: one
+# element, one short of a tile, one over, and several tiles of each kind.  `spread`
+# scales rows and columns by up to 10^+-spread, past the range in which the scaled
+# value is formed from float pairs (spread 12: factors near 1e-12 on values near 1e24).
+# 64 iterations in FP32 products as in test_shared_iterates_match_oracle: 1e-5.
+@pytest.mark.parametrize("m,n,spread", [(1, 1, 0), (63, 255, 0), (65, 257, 0), (64, 1024, 0),
+                                        (130, 1028, 3), (70, 515, 12)])
+def test_shared_scaling_tiles_match_oracle(C, m, n, spread):
+    rng = np.random.default_rng(m * 1000 + n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    A[rng.random((m, n)) < 0.1] = 0.0
+    A *= 10.0 ** rng.uniform(-spread, spread, (m, 1)) * 10.0 ** rng.uniform(-spread, spread, n)
+    A = A.astype(np.float32)
+    A64 = A.astype(np.float64)
+    x0 = rng.uniform(0, 1, n)
+    b, c = A64 @ x0, A64.T @ (rng.standard_normal((2, m)) / np.maximum(np.abs(A64).max(1), 1e-300)).T
+    p = O.Problem(sp.csr_matrix(A64), c[:, 1].copy(), b, b, np.zeros(n), np.ones(n))
+    opts = dict(eps_abs=1e-14, eps_rel=1e-14, iteration_limit=64, power_max_iter=0)
+    ref = O.solve_lp(p, O.Options(eps_primal_infeasible=0.0, eps_dual_infeasible=0.0, **opts))
+    h = C.mpax_lp_shared_create(m, n, 2, A, np.ascontiguousarray(c.T), b, b, np.zeros(n), np.ones(n))
+    try:
+        C.mpax_shared_solve(h, C.mpax_options_default(fp64_continuation=0, **opts), True)
+        X, Y = C.mpax_shared_get_solution(h, m, n, 2)
+    finally:
+        C.mpax_shared_destroy(h)
+    # in the scaled space, where every coordinate has the same weight
+    assert rel_inf(X[1] / ref.Dc, ref.x / ref.Dc) <= 1e-5
+    assert rel_inf(Y[1] / ref.Dr, ref.y / ref.Dr) <= 1e-5
