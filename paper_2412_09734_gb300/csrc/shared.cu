@@ -714,19 +714,96 @@ __global__ void k_bound_norm(const double* lc, const double* uc, const double* D
   }
 }
 
-__global__ void k_vec_norm_part(const float* __restrict__ v, size_t n, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double s = 0;
-  for (size_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)v[i] * (double)v[i];
+// ---- power iteration for ||A~||_2 on the device ------------------------------------
+// A round is w = A~ v, g = A~^T w (the matrix-vector kernels below), v = g / ||g||; its
+// norm, stop rule and estimate stay on the device, so the host reads the state once
+// every kPowerBatch rounds.  Rounds launched past the last return at once.
+// Bound by the two reads of A per round (0.54 GB at 8192 x 16384: 80 us each); with the
+// norm in one block, the rescaling and a host round trip per round a round took 205 us.
+constexpr int kPowerBatch = 8;
+constexpr int kPowerBlocks = 512;  // at most: every block of k_power_scale adds all partials
+struct PowerState {
+  double nu, prev, d_prev;
+  int done;    // the round that ended the iteration, 0 while it runs
+  int rounds;  // rounds taken
+};
+
+// Sum of the block partials part[0..nb) in a fixed order, returned to every thread.
+__device__ __forceinline__ double sum_to_all(const double* __restrict__ part, int nb, double* sh) {
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) s += part[b];
   s = block_sum(s, sh);
-  if (threadIdx.x == 0) *out = sqrt(s);
+  __shared__ double all;
+  if (threadIdx.x == 0) all = s;
+  __syncthreads();
+  return all;
 }
 
-__global__ void k_scale_f(float* __restrict__ v, size_t n, const double* __restrict__ nrm) {
-  const double inv = *nrm > 0 ? 1.0 / *nrm : 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    v[i] = (float)((double)v[i] * inv);
+// Start vector (power_start_raw): squares per block, then v = raw / ||raw||.
+__global__ void k_power_start_sq(int n, double* __restrict__ part, PowerState* st) {
+  __shared__ double sh[32];
+  const int j0 = blockIdx.x * blockDim.x + threadIdx.x;
+  double q = 0.0;
+  for (int j = j0; j < n; j += gridDim.x * blockDim.x) {
+    const double r = power_start_raw(j);
+    q += r * r;
+  }
+  const double s = block_sum(q, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (j0 == 0) *st = PowerState{0.0, 0.0, 0.0, 0, 0};
+}
+__global__ void k_power_start_vec(int n, const double* __restrict__ part, float* __restrict__ v) {
+  __shared__ double sh[32];
+  const double ss = sum_to_all(part, gridDim.x, sh);
+  const double inv = 1.0 / sqrt(ss > 0.0 ? ss : 1.0);
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    v[j] = (float)(power_start_raw(j) * inv);
+}
+
+// g_j = the sum of the product's chunk partials in order; squares of g per block.
+__global__ void k_power_sum(const float* __restrict__ gpart, int chunks, int n,
+                            float* __restrict__ g, double* __restrict__ part,
+                            const PowerState* st) {
+  __shared__ double sh[32];
+  if (st->done) return;
+  double q = 0.0;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    float t = 0.0f;
+#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) t += gpart[(size_t)c * n + j];
+    g[j] = t;
+    q += (double)t * (double)t;
+  }
+  const double s = block_sum(q, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+// End of round t: v = g / ||g||, and in block 0 the stop rule (power_stop) and the
+// estimate.  A block that already sees this round's `done` may skip its part of v,
+// which no later round reads.
+__global__ void k_power_scale(float* __restrict__ v, int n, const double* __restrict__ part,
+                              PowerState* st, int t, int max_iter, double tol, double cap) {
+  __shared__ double sh[32];
+  if (st->done) return;
+  const double nrm = sqrt(sum_to_all(part, gridDim.x, sh));
+  const double inv = nrm > 0 ? 1.0 / nrm : 0.0;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    v[j] = (float)((double)v[j] * inv);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->rounds = t;
+    if (nrm == 0.0) {  // the previous estimate stands
+      st->done = t;
+      return;
+    }
+    double nu = sqrt(nrm), est = nu, d = st->d_prev;
+    bool stop = t > 1 && power_stop(nu, st->prev, &d, tol, cap, &est);
+    if (stop) nu = est;
+    else if (t == max_iter && isfinite(cap)) nu = cap;
+    st->d_prev = d;
+    st->prev = nu;
+    st->nu = nu;
+    if (stop || t == max_iter) st->done = t;
+  }
 }
 
 // SPO+ (Sec. 3.4): c' = 2 c_hat - c_true; per instance k (one block),
@@ -783,6 +860,8 @@ struct mpax_shared {
   float2 *fr = nullptr, *fc = nullptr;    // scaling factors of a pass as float pairs
   unsigned* nmax = nullptr;               // row then column maxima of a Ruiz round
   int ctiles = 1;                         // column tiles of a scaling pass
+  PowerState* pstate = nullptr;           // power iteration: state and block partials
+  double* ppart = nullptr;
   float4* step = nullptr;                 // per-instance step sizes (k_coefs)
   float2* halpern = nullptr;              // Halpern weights of kCoefIters iterations (k_coefs)
   int chunks = 1;                         // chunks of the check reductions
@@ -833,7 +912,7 @@ void free_shared(mpax_shared* sh) {
                   sh->yprev, sh->xh_hi, sh->xh_lo, sh->y_hi, sh->y_lo, sh->part, sh->cn,
                   sh->cns, sh->inst, sh->Xout, sh->Yout, sh->gpart, sh->gpart_n, sh->spo,
                   sh->uerr, sh->iDr, sh->iDc, sh->step, sh->halpern, sh->fr, sh->fc,
-                  sh->nmax};
+                  sh->nmax, sh->pstate, sh->ppart};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (sh->s) cudaStreamDestroy(sh->s);
@@ -860,7 +939,9 @@ template <int V>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv_t_part(const float* __restrict__ A, int m,
                                                               int n, const float* __restrict__ y,
                                                               int rows_per,
-                                                              float* __restrict__ part) {
+                                                              float* __restrict__ part,
+                                                              const int* skip) {
+  if (skip && *skip) return;
   const int j0 = (blockIdx.x * kGemvThreads + threadIdx.x) * V;
   if (j0 >= n) return;
   const int r0 = blockIdx.y * rows_per, r1 = min(m, r0 + rows_per);
@@ -903,7 +984,8 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_t_part(const float* __res
 
 // T_j = sum_s part[s][j], s in order.
 __global__ void k_gemv_t_sum(const float* __restrict__ part, int chunks, int n,
-                             float* __restrict__ T) {
+                             float* __restrict__ T, const int* skip = nullptr) {
+  if (skip && *skip) return;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
     float t = 0.0f;
     for (int c = 0; c < chunks; ++c) t += part[(size_t)c * n + j];
@@ -921,7 +1003,9 @@ template <int V>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv_n_part(const float* __restrict__ A, int m,
                                                               int n, const float* __restrict__ w,
                                                               int cols_per,
-                                                              float* __restrict__ part) {
+                                                              float* __restrict__ part,
+                                                              const int* skip) {
+  if (skip && *skip) return;
   constexpr int R = kGemvRows;
   __shared__ float sh[R][kGemvThreads / 32];
   const int r0 = blockIdx.x * R;
@@ -1092,22 +1176,24 @@ namespace {
 using namespace mpax_gemv;
 
 // B = 1, FP32 products: the partial-sum kernel of one product, trans = 1: A v
-// into gpart_n (column chunks), trans = 0: A^T v into gpart (row chunks).
-void gemv_part(mpax_shared* sh, int trans, const float* vf, const float* Mf) {
+// into gpart_n (column chunks), trans = 0: A^T v into gpart (row chunks).  A set
+// device flag *skip (nullable) turns the launch into a no-op.
+void gemv_part(mpax_shared* sh, int trans, const float* vf, const float* Mf,
+               const int* skip = nullptr) {
   const int m = sh->m, n = sh->n;
   const bool v4 = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(Mf) & 15) == 0) &&
                   ((reinterpret_cast<uintptr_t>(vf) & 15) == 0);
   if (trans) {
     const dim3 grid((m + kGemvRows - 1) / kGemvRows, sh->gemv_nchunks);
     const int cols_per = ((n + sh->gemv_nchunks - 1) / sh->gemv_nchunks + 3) / 4 * 4;
-    if (v4) k_gemv_n_part<4><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, cols_per, sh->gpart_n);
-    else k_gemv_n_part<1><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, cols_per, sh->gpart_n);
+    if (v4) k_gemv_n_part<4><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, cols_per, sh->gpart_n, skip);
+    else k_gemv_n_part<1><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, cols_per, sh->gpart_n, skip);
   } else {
     const int V = v4 ? 4 : 1;
     const dim3 grid((n + V * kGemvThreads - 1) / (V * kGemvThreads), sh->gemv_chunks);
     const int rows_per = (m + sh->gemv_chunks - 1) / sh->gemv_chunks;
-    if (v4) k_gemv_t_part<4><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, rows_per, sh->gpart);
-    else k_gemv_t_part<1><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, rows_per, sh->gpart);
+    if (v4) k_gemv_t_part<4><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, rows_per, sh->gpart, skip);
+    else k_gemv_t_part<1><<<grid, kGemvThreads, 0, sh->s>>>(Mf, m, n, vf, rows_per, sh->gpart, skip);
   }
   sh->gemv_launches += 1;
   sh->gemms += 1;
@@ -1307,6 +1393,8 @@ mpax_status mpax_lp_shared_create(int32_t m, int32_t n, int32_t B, const float* 
   al(&sh->fr, m);
   al(&sh->fc, n);
   al(&sh->nmax, (size_t)m + n);
+  al(&sh->pstate, 1);
+  al(&sh->ppart, kPowerBlocks);
   al(&sh->step, B);
   al(&sh->halpern, (size_t)kCoefIters * B);
   al(&sh->cn, B);
@@ -1422,40 +1510,34 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   {
     float* v = sh->T;    // n (first column of T as scratch)
     float* wv = sh->S;   // m
-    std::vector<float> v0(n);  // the common start vector (power_start_raw), normalised
-    double ss = 0.0;
-    for (int j = 0; j < n; ++j) ss += power_start_raw(j) * power_start_raw(j);
-    const double inv = 1.0 / std::sqrt(ss > 0.0 ? ss : 1.0);
-    for (int j = 0; j < n; ++j) v0[j] = (float)(power_start_raw(j) * inv);
-    cudaMemcpyAsync(v, v0.data(), sizeof(float) * n, cudaMemcpyHostToDevice, s);
-    double prev = 0.0, nu = 0.0, d_prev = 0.0;
-    sh->power_rounds = 0;
-    for (int t = 1; t <= o->power_max_iter; ++t) {
-      sh->power_rounds = t;
-      // wv = A~ v, v = A~^T wv with this file's matrix-vector kernels
-      gemv_part(sh, 1, v, sh->As);
-      k_gemv_t_sum<<<g1(m), 256, 0, s>>>(sh->gpart_n, sh->gemv_nchunks, m, wv);
-      gemv_part(sh, 0, wv, sh->As);
-      k_gemv_t_sum<<<g1(n), 256, 0, s>>>(sh->gpart, sh->gemv_chunks, n, v);
-      k_vec_norm_part<<<1, 512, 0, s>>>(v, n, sh->scal);
-      double nrm = 0.0;
-      cudaMemcpyAsync(&nrm, sh->scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-      cudaStreamSynchronize(s);
-      k_scale_f<<<g1(n), 256, 0, s>>>(v, n, sh->scal);
-      L += 4;
-      if (nrm == 0.0) break;
-      nu = std::sqrt(nrm);
-      double est = nu;
-      const double cap = o->pock_chambolle ? 1.0 : INFINITY;
-      if (t > 1 && power_stop(nu, prev, &d_prev, o->power_tol, cap, &est)) {
-        nu = est;
-        break;
-      }
-      if (t == o->power_max_iter && std::isfinite(cap)) nu = cap;
-      prev = nu;
+    const int nb = std::min(kPowerBlocks, (n + 255) / 256);
+    const double cap = o->pock_chambolle ? 1.0 : INFINITY;
+    const int* skip = &sh->pstate->done;
+    PowerState ps{};
+    if (o->power_max_iter > 0) {
+      k_power_start_sq<<<nb, 256, 0, s>>>(n, sh->ppart, sh->pstate);
+      k_power_start_vec<<<nb, 256, 0, s>>>(n, sh->ppart, v);
+      L += 2;
     }
-    if (o->power_max_iter == 0) nu = 1.0;  // the bound of the Pock-Chambolle round
-    sh->norm_A = nu;
+    for (int t = 1; t <= o->power_max_iter; ++t) {
+      // wv = A~ v, v = A~^T wv with this file's matrix-vector kernels
+      gemv_part(sh, 1, v, sh->As, skip);
+      if (sh->gemv_nchunks > 1) {
+        k_gemv_t_sum<<<g1(m), 256, 0, s>>>(sh->gpart_n, sh->gemv_nchunks, m, wv, skip);
+        L += 1;
+      }
+      gemv_part(sh, 0, sh->gemv_nchunks > 1 ? wv : sh->gpart_n, sh->As, skip);
+      k_power_sum<<<nb, 256, 0, s>>>(sh->gpart, sh->gemv_chunks, n, v, sh->ppart, sh->pstate);
+      k_power_scale<<<nb, 256, 0, s>>>(v, n, sh->ppart, sh->pstate, t, o->power_max_iter,
+                                       o->power_tol, cap);
+      L += 2;
+      if (t % kPowerBatch == 0 || t == o->power_max_iter) {
+        cudaMemcpyAsync(&ps, sh->pstate, sizeof(ps), cudaMemcpyDeviceToHost, s);
+        if (cudaStreamSynchronize(s) != cudaSuccess || ps.done) break;
+      }
+    }
+    sh->power_rounds = ps.rounds;
+    sh->norm_A = o->power_max_iter == 0 ? 1.0 : ps.nu;  // 1: the Pock-Chambolle bound
   }
   const double eta = sh->norm_A > 0 ? o->step_safety / sh->norm_A : 1.0;
   cudaStreamSynchronize(s);
