@@ -37,6 +37,7 @@
 #include "../../include/mpax.h"
 #include "umma_host.h"
 #include "common.cuh"
+#include "sgemm.cuh"
 
 namespace mpax {
 
@@ -1051,124 +1052,6 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_n_part(const float* __res
   }
 }
 
-// ---- B > 1, FP32 products on the CUDA cores ----------------------------------------
-// C[n][m] = sum_k A_op[m][k] V[n][k] for the B instances' vectors V (rows of ldv):
-// A_op = A~ stored [M][K] (A_MN = 0, the dual step's A~ X) or A~^T of an A~ stored
-// [K][M] (A_MN = 1, the primal step's A~^T Y).  CTA tile 128 (M) x 128 (N) x 8 (K),
-// 256 threads of 8 x 8 outputs each, accumulated in FP32 in increasing k (one
-// fixed order per output).  The next k-slab is read from global memory into
-// registers while the current one is multiplied, then stored into the other of
-// two shared-memory buffers (one barrier per slab).
-constexpr int kSgBM = 128, kSgBN = 128, kSgBK = 8;
-
-template <int A_MN>
-__device__ __forceinline__ void sg_load_a(const float* __restrict__ A, long long lda, int M, int K,
-                                          int m0, int k0, int tid, float* ra) {
-  // 128 x 8 values, 4 per thread
-  if (A_MN) {  // rows k0..k0+7 of 128 contiguous m values: thread -> (k, 4 m)
-    const int kk = tid / 32, mm = (tid % 32) * 4;
-    const int gk = k0 + kk;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int gm = m0 + mm + t;
-      ra[t] = (gk < K && gm < M) ? A[(long long)gk * lda + gm] : 0.0f;
-    }
-  } else {     // 128 rows m of 8 contiguous k values: thread -> (m, 4 k)
-    const int r = tid / 2, kq = (tid % 2) * 4;
-    const int gm = m0 + r;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int gk = k0 + kq + t;
-      ra[t] = (gm < M && gk < K) ? A[(long long)gm * lda + gk] : 0.0f;
-    }
-  }
-}
-
-template <int A_MN>
-__device__ __forceinline__ void sg_store_a(float (*As)[kSgBM + 4], int tid, const float* ra) {
-  if (A_MN) {
-    const int kk = tid / 32, mm = (tid % 32) * 4;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) As[kk][mm + t] = ra[t];
-  } else {
-    const int r = tid / 2, kq = (tid % 2) * 4;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) As[kq + t][r] = ra[t];
-  }
-}
-
-template <int A_MN>
-__global__ void __launch_bounds__(256) k_sgemm(const float* __restrict__ A, long long lda,
-                                               const float* __restrict__ V, long long ldv,
-                                               float* __restrict__ Cm, long long ldc, int M,
-                                               int N, int K) {
-  __shared__ __align__(16) float As[2][kSgBK][kSgBM + 4];
-  __shared__ __align__(16) float Vs[2][kSgBK][kSgBN + 4];
-  const int tid = threadIdx.x;
-  const int tm = tid % 16, tn = tid / 16;  // 8 rows (m) and 8 instances (n) each
-  const int m0 = blockIdx.x * kSgBM, n0 = blockIdx.y * kSgBN;
-  float acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-  // V slab: 128 rows n of 8 contiguous k values: thread -> (n, 4 k)
-  const int vr = tid / 2, vq = (tid % 2) * 4;
-  float ra[4], rv[4];
-  auto load_v = [&](int k0) {
-    const int gn = n0 + vr;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int gk = k0 + vq + t;
-      rv[t] = (gn < N && gk < K) ? V[(long long)gn * ldv + gk] : 0.0f;
-    }
-  };
-  sg_load_a<A_MN>(A, lda, M, K, m0, 0, tid, ra);
-  load_v(0);
-  sg_store_a<A_MN>(As[0], tid, ra);
-#pragma unroll
-  for (int t = 0; t < 4; ++t) Vs[0][vq + t][vr] = rv[t];
-  __syncthreads();
-  int buf = 0;
-  for (int k0 = 0; k0 < K; k0 += kSgBK) {
-    const bool more = k0 + kSgBK < K;
-    if (more) {
-      sg_load_a<A_MN>(A, lda, M, K, m0, k0 + kSgBK, tid, ra);
-      load_v(k0 + kSgBK);
-    }
-#pragma unroll
-    for (int kk = 0; kk < kSgBK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][tm * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][tm * 8 + 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Vs[buf][kk][tn * 8]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Vs[buf][kk][tn * 8 + 4]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    if (more) {
-      sg_store_a<A_MN>(As[buf ^ 1], tid, ra);
-#pragma unroll
-      for (int t = 0; t < 4; ++t) Vs[buf ^ 1][vq + t][vr] = rv[t];
-    }
-    __syncthreads();
-    buf ^= 1;
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int gn = n0 + tn * 8 + j;
-    if (gn >= N) continue;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int gm = m0 + tm * 8 + i;
-      if (gm < M) Cm[(long long)gn * ldc + gm] = acc[i][j];
-    }
-  }
-}
-
 }  // namespace mpax_gemv
 
 namespace {
@@ -1251,12 +1134,10 @@ cudaError_t product_impl(mpax_shared* sh, int trans, const __nv_bfloat16* vhi,
   if (!bf16x3) {
     // FP32 on the CUDA cores: trans = 1 is A~ V (A~ [m][n] K-major), trans = 0
     // is A~^T V (the same storage read M-major)
-    const dim3 grid((rows + kSgBM - 1) / kSgBM, (B + kSgBN - 1) / kSgBN);
-    if (trans) k_sgemm<0><<<grid, 256, 0, sh->s>>>(Mf, n, vf, K, C, rows, rows, B, K);
-    else k_sgemm<1><<<grid, 256, 0, sh->s>>>(Mf, n, vf, K, C, rows, rows, B, K);
     sh->gemms += 1;
     sh->gemm_flops += 2.0 * rows * (double)B * K;
-    return cudaGetLastError();
+    return trans ? sgemm<0>(Mf, n, vf, K, C, rows, rows, B, K, sh->s)
+                 : sgemm<1>(Mf, n, vf, K, C, rows, rows, B, K, sh->s);
   }
   // A_hi V_lo + A_lo V_hi + A_hi V_hi in one tensor-core kernel (umma.cuh); the
   // plan of this direction holds the split buffers (vhi, vlo) and the output C

@@ -270,3 +270,24 @@ def test_shared_scaling_tiles_match_oracle(C, m, n, spread):
     # in the scaled space, where every coordinate has the same weight
     assert rel_inf(X[1] / ref.Dc, ref.x / ref.Dc) <= 1e-5
     assert rel_inf(Y[1] / ref.Dr, ref.y / ref.Dr) <= 1e-5
+
+
+# The FP32 products pick a tile by the size of the grid: 32 x 32 outputs, 64 x 32 from 128
+# tiles on, 128 x 128 from 100 of those on; each with partial tiles in every dimension.
+# Tolerance as above (64 iterations of FP32 products: 1e-5).
+@pytest.mark.parametrize("m,n,B", [(33, 71, 35), (1290, 1301, 199), (1281, 1290, 1250)],
+                         ids=["32x32", "64x32", "128x128"])
+def test_shared_fp32_product_tiles_match_oracle(C, m, n, B):
+    d = shared_dense_lp_batch(m, n, B, seed=m + B, bound_frac=0.5)
+    opts = dict(eps_abs=1e-14, eps_rel=1e-14, iteration_limit=64, power_max_iter=0)
+    h = C.mpax_lp_shared_create(m, n, B, d["A"], d["C"], d["b"], d["b"], d["l"], d["u"])
+    try:
+        C.mpax_shared_solve(h, C.mpax_options_default(fp64_continuation=0, **opts), True)
+        X, Y = C.mpax_shared_get_solution(h, m, n, B)
+    finally:
+        C.mpax_shared_destroy(h)
+    for k in (0, B // 2, B - 1):
+        ref = O.solve_lp(_oracle_problem(d, k), O.Options(
+            eps_primal_infeasible=0.0, eps_dual_infeasible=0.0, **opts))
+        assert rel_inf(X[k], ref.x) <= 1e-5, k
+        assert rel_inf(Y[k], ref.y) <= 1e-5, k
