@@ -64,6 +64,12 @@ constexpr int kBU = MPAX_BATCH_UNROLL;
 #define MPAX_BATCH_SMEM_RP 1
 #endif
 
+// Iterations whose Halpern weights the CTA forms at a time.  A double-precision division
+// takes tens of instructions, each 16 cycles of the SM's FP64 pipe per warp, so the
+// weights are formed by one warp or two for 64 iterations and not by every thread in
+// each: @FIG@.
+constexpr int kCoefs = 64;
+
 template <typename T>
 struct BatchArgs {
   int B;
@@ -76,7 +82,7 @@ struct BatchArgs {
   const int* colt;
   const T* valt;
   const T *c, *l, *u, *lc, *uc;                 // scaled data
-  const double *c0, *l0, *u0, *lc0, *uc0, *Dr, *Dc;  // originals and scaling
+  const double *c0, *l0, *u0, *lc0, *uc0, *Dr, *Dc, *iDr, *iDc;  // originals, scaling, inverses
   T *w, *xa, *xhat, *ya, *yhat, *gbuf;          // iterate storage
   double *xout, *yout;
   int* status;
@@ -225,6 +231,7 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
                                                unsigned long long t_launch) {
   const unsigned long long t_start = gtimer();
   __shared__ int s_late;
+  __shared__ T s_coef[kCoefs + 1];
   const int m0 = (int)a.m_off[b], mb = (int)(a.m_off[b + 1] - a.m_off[b]);
   const int n0 = (int)a.n_off[b], nb = (int)(a.n_off[b + 1] - a.n_off[b]);
   const int grp = threadIdx.x / kLPR, gl = threadIdx.x % kLPR;
@@ -380,8 +387,13 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
     const T tt = (T)tau, ss = (T)sigma, iss = (T)(1.0 / sigma);
     for (int it = 0; it < len; ++it) {
       const bool chk = (it == len - 1);
-      const T rb = (T)(1.0 / (double)(k + 1));  // rebuild weight of x^{n,k}
-      const T hb = (T)(1.0 / (double)(k + 2));  // Halpern weight of the anchor
+      // weights 1/(k+1) and 1/(k+2) of this and the next iterations
+      if (it % kCoefs == 0) {
+        if (threadIdx.x <= min(kCoefs, len - it)) s_coef[threadIdx.x] = (T)(1.0 / (double)(k + 1 + threadIdx.x));
+        __syncthreads();
+      }
+      const T rb = s_coef[it % kCoefs];      // rebuild weight of x^{n,k}
+      const T hb = s_coef[it % kCoefs + 1];  // Halpern weight of the anchor
       // primal half-step over the rows of A^T (eq. 3, first line).  Each kLPR-lane
       // group takes kBR rows per step (j, j + G, ...) and issues the row pointers,
       // the epilogue operands and both rows' products before reducing, so every
@@ -487,7 +499,7 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
       s = group_sum(s);
       if (gl == 0 && in_i) {
         const int g = m0 + i;
-        const double ax = (double)s / a.Dr[g];
+        const double ax = (double)s * a.iDr[g];
         const double lo = a.lc0[g], hi = a.uc0[g];
         const double r = ax - fmin(fmax(ax, lo), hi);
         K0 += r * r;
@@ -505,7 +517,7 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
       s = group_sum(s);
       if (gl == 0 && in_j) {
         const int g = n0 + j;
-        const double aty = (double)s / a.Dc[g];
+        const double aty = (double)s * a.iDc[g];
         const double x = a.Dc[g] * (double)xs[j];
         const double lam = a.c0[g] - aty;
         const double lo = a.l0[g], hi = a.u0[g];
@@ -845,6 +857,8 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
   a.uc0 = P.uc;
   a.Dr = P.Dr;
   a.Dc = P.Dc;
+  a.iDr = P.invDr;
+  a.iDc = P.invDc;
   a.w = w;
   a.xa = xa;
   a.xhat = xhat;
