@@ -281,7 +281,7 @@ mpax_status create_common(int32_t m, int32_t n, int64_t nnz, const int64_t* row_
   if (!e) e = dmalloc(&P.rowred2, m);
   if (!e) e = dmalloc(&P.colred2, n);
   // (also the 32-bin row-length histogram of the kernel autotuner)
-  if (!e) e = dmalloc(&P.tmp_rows, std::max<size_t>(big, 64));
+  if (!e) e = dmalloc(&P.tmp_rows, std::max<size_t>(2 * (size_t)big + 2, 64));
   if (!e) e = dmalloc(&P.tmp_scan, scan_tmp_ints(big));
   if (!e) e = dmalloc(&P.red, kRedBlocks * 8);
   if (!e) e = dmalloc(&P.red_out, 16);
@@ -420,11 +420,13 @@ mpax_status do_prepare(mpax_problem* pb, const mpax_options* o, long long* launc
   cudaStream_t s = P.s;
   if (P.is_qp && o->power_max_iter == 0)
     return fail(MPAX_ERR_INVALID_ARGUMENT, "power_max_iter = 0 is for LPs (||Q~|| has no bound)");
-  // structure: transpose(s) and work-item schedules
-  TRY_CUDA(transpose_csr(P.A, P.At, P.permT, P.tmp_rows, P.tmp_scan, s), "transpose");
+  // structure: transpose(s) and work-item schedules (the scaled values, rewritten by the
+  // scaling below, are the transposes' scratch)
+  TRY_CUDA(transpose_csr(P.A, P.At, P.permT, P.tmp_rows, P.tmp_scan, P.val_s, s), "transpose");
   *launches += 6;
   if (P.is_qp) {
-    TRY_CUDA(transpose_csr(P.F, P.Ft, P.permF, P.tmp_rows, P.tmp_scan, s), "transpose F");
+    TRY_CUDA(transpose_csr(P.F, P.Ft, P.permF, P.tmp_rows, P.tmp_scan, P.fval_s, s),
+             "transpose F");
     *launches += 6;
   }
   P.transposed = true;

@@ -1094,7 +1094,7 @@ mpax_status mpax_batch_solve(mpax_batch* bt, const mpax_options* o) {
   cudaStream_t s = P.s;
   problem_order_after_user(bt->prob);
   long long launches = 0;
-  cudaError_t e = transpose_csr(P.A, P.At, P.permT, P.tmp_rows, P.tmp_scan, s);
+  cudaError_t e = transpose_csr(P.A, P.At, P.permT, P.tmp_rows, P.tmp_scan, P.val_s, s);
   if (!e) e = compute_scaling(P, o->ruiz_iters, o->pock_chambolle != 0);
   launches += 6 + 5 * o->ruiz_iters + 8;
   if (e) return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));

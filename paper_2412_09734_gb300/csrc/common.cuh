@@ -262,9 +262,10 @@ extern unsigned long long sched_generation;
 // (the L2 bulk prefetch rounds its range out to 16 bytes).
 constexpr int kPad = 16;
 
-// Device transpose: At.rp/At.col/perm allocated by the caller (n+1, nnz, nnz).
+// Device transpose: At.rp/At.col/perm allocated by the caller (n+1, nnz, nnz); tmp_nnz:
+// nnz scratch elements.
 cudaError_t transpose_csr(const Csr& A, Csr& At, int* perm, int* tmp_cnt, int* tmp_scan,
-                          cudaStream_t s);
+                          double* tmp_nnz, cudaStream_t s);
 
 }  // namespace mpax
 

@@ -52,7 +52,7 @@ struct ProblemData {
   double* colred2 = nullptr;  // n work
 
   // scratch
-  int* tmp_rows = nullptr;    // max(m, n, r) + 2 ints
+  int* tmp_rows = nullptr;    // 2 (max(m, n, r) + 2) ints
   int* tmp_scan = nullptr;    // scan_tmp_ints(max(m, n, r) + 1)
   double* red = nullptr;      // reduction partials (kRedBlocks * 8)
   double* red_out = nullptr;  // 16 doubles
