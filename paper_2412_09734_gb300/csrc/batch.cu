@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/mpax.h"
@@ -26,48 +27,25 @@
 
 namespace mpax {
 
-// Threads of the CTA that solves one instance, and CTAs per SM at 64 registers a
-// thread.  Measured on 4,096 instances of the bench recipe: FP32 1024 threads 0.323 s
-// per batch (instance p50 6.5 ms), 512 threads 0.334 s (11.8 ms), 256 threads
-// 0.435 s; FP64 512 threads 0.461 s, 1024 threads 0.488 s, 256 threads 0.80 s.
+// Threads of the CTA that solves one instance, one CTA per SM.  FP32: 1024 at 64 registers
+// (2,000 instances of 50 to 2,000 rows 56 ms; two CTAs of 512 71 ms); FP64: 512 at 128
+// registers (300 of them 33 ms; two CTAs of 512 at 64 registers, which spill, 40 ms).
 template <typename T>
 constexpr int kBatchThreads = sizeof(T) == 4 ? 1024 : 512;
 template <typename T>
-constexpr int kBatchMinB = 1024 / kBatchThreads<T>;
+constexpr int kBatchMinB = 1;
 constexpr double kBatchMaxSeconds = 600.0;
-// Lanes cooperating on one row of an instance (a power of two <= 32).  Rows of
-// the batch recipe hold ~1-40 nonzeros: measured on 4096 instances, 2 lanes per
+// Partial sums of a row: entries 0, 2, 4, ... and 1, 3, 5, ..., added at the end.  In CSR
+// (RowsCsr) two lanes hold them.  Rows of the batch recipe hold ~1-40 nonzeros: measured on 4096 instances, 2 lanes per
 // row (0.325 s per batch mixed, 0.450 s FP64) beat 8 (0.490 / 0.956 s) and 1
 // (0.521 / 0.597 s) -- with 8 lanes a row's shuffle reduction and its one-lane
 // epilogue cost more than its two or three loads per lane.
-#ifndef MPAX_BATCH_LPR
-#define MPAX_BATCH_LPR 2
-#endif
-constexpr int kLPR = MPAX_BATCH_LPR;
-// Rows each lane group carries per step of a half-step (their memory round
-// trips overlap).  With 2-lane groups a step already covers 256 rows, and 1 row
-// per group measured best (0.325 against 0.329 s per 4096-instance batch).
-#ifndef MPAX_BATCH_ROWS
-#define MPAX_BATCH_ROWS 1
-#endif
-constexpr int kBR = MPAX_BATCH_ROWS;
-// Values and columns each lane loads per row before using any (see rows_dot).
-// Measured on 1024 instances of the bench recipe: 1 (0.369 s per batch, mixed)
-// beats 2 (0.370 s) and 4 (0.405 s): at 64 registers deeper batches spill.
-#ifndef MPAX_BATCH_UNROLL
-#define MPAX_BATCH_UNROLL 1
-#endif
-constexpr int kBU = MPAX_BATCH_UNROLL;
-// 1: stage each instance's row pointers in shared memory when two CTAs per SM
-//    still fit (<= 100 KB of shared memory per CTA).
-#ifndef MPAX_BATCH_SMEM_RP
-#define MPAX_BATCH_SMEM_RP 1
-#endif
-
+constexpr int kLPR = 2;
 // Iterations whose Halpern weights the CTA forms at a time.  A double-precision division
 // takes tens of instructions, each 16 cycles of the SM's FP64 pipe per warp, so the
 // weights are formed by one warp or two for 64 iterations and not by every thread in
-// each: @FIG@.
+// each (512 ragged LPs, FP32: the launch 38.4 -> 35.2 ms together with reciprocal
+// scaling factors in the checks; 64 grid LPs in FP64: an iteration 13.3 -> 11.9 us).
 constexpr int kCoefs = 64;
 
 template <typename T>
@@ -90,14 +68,20 @@ struct BatchArgs {
   long long* restarts;
   double *relkkt, *pobj, *secs;
   int* next;
+  // Rows by length (k_sort_rows): the vectors and scaled data of an instance lie in its
+  // sorted order; permm / permn give the original (local) index.  An instance whose zs
+  // range is empty keeps the original order and the CSR arrays above.
+  const int *permm, *permn;
+  const unsigned short *lenm, *lenn;   // row lengths, sorted order
+  const int *soffm, *soffn;            // slice offsets; instance b's start at slice_base
+  const long long *zsa, *zst;          // B + 1: storage of the sorted matrices
+  const T *sval, *svalt;
+  const unsigned short *scol, *scolt;  // sorted local indices of the gathered vector
   // Shared-memory pool of a CTA: smem_vec elements for the instance's two
-  // gathered vectors (y, m_b entries, then the primal vector, n_b entries) and
-  // then rp_cap ints for its row pointers.  An instance with m_b + n_b >
-  // smem_vec keeps both vectors in global memory instead (gys, gxs: its slices
-  // of two m- and n-vectors); one with m_b + n_b + 2 > rp_cap reads its row
-  // pointers in place.
+  // gathered vectors (y, m_b entries, then the primal vector, n_b entries).  An instance
+  // with m_b + n_b > smem_vec keeps both vectors in global memory instead (gys, gxs: its
+  // slices of two m- and n-vectors).
   int smem_vec;
-  int rp_cap;
   T* gys;
   T* gxs;
   double eps_abs, eps_rel, r_suff, r_nec, r_art, pw_smooth, step_safety, power_tol;
@@ -143,80 +127,140 @@ __device__ __forceinline__ unsigned long long gtimer() {
   return t;
 }
 
-// Dot products of kBR rows (one per slot r, lane offset already in pp[r]) with
-// the shared-memory vector vec (columns offset by off): each pass issues up to
-// kBU values and columns per row and lane before any of them is used, so a row
-// of up to kBU * kLPR nonzeros costs one memory round trip.
+// ---- the rows of one matrix of an instance ----------------------------------------
+// each(vec, pre, row): for every row i, s = the row times vec; pre(i) is called before the
+// row's loads (it returns the operands of row's epilogue, which travel with them) and
+// row(i, s, operands) on one thread after.
+
+// CSR, two lanes per row: for instances whose vectors do not fit in shared memory or
+// whose rows are too uneven to sort.
 template <typename T>
-__device__ __forceinline__ void rows_dot(const int* pp, const int* pe, const T* __restrict__ val,
-                                         const int* __restrict__ col, const T* vec, int off,
-                                         T* sr) {
-  for (int base = 0;; base += kBU * kLPR) {
-    T v[kBR][kBU];
-    int c[kBR][kBU];
-    bool any = false;
+struct RowsCsr {
+  int rows;
+  const int* rp;
+  const T* val;
+  const int* col;
+  int off;  // columns are global: less off
+  template <class Pre, class Row>
+  __device__ __forceinline__ void each(const T* vec, Pre pre, Row row) const {
+    const int grp = threadIdx.x / kLPR, gl = threadIdx.x % kLPR;
+    const int G = blockDim.x / kLPR;
+    for (int i0 = 0; i0 < rows; i0 += G) {
+      const int i = i0 + grp;
+      const bool in = i < rows;
+      const int pe = in ? rp[i + 1] : 0;
+      decltype(pre(0)) q{};
+      if (gl == 0 && in) q = pre(i);
+      T s = 0;
+      for (int p = in ? rp[i] + gl : 0; p < pe; p += kLPR) s += val[p] * vec[col[p] - off];
+      s = group_sum(s);
+      if (gl == 0 && in) row(i, s, q);
+    }
+  }
+};
+
+// Rows sorted by length, longest first, in slices of 32 stored entry-major: a thread per
+// row, so that a warp's loads of values and 16-bit columns are consecutive, its epilogues
+// use every lane (an FP64 instruction costs the same 16 cycles for one lane as for 32)
+// and rows of a warp end together.  In CSR with two lanes per row a warp load touched
+// 16 rows' sectors and every second lane idled in the epilogue: 2.7 warp instructions per
+// nonzero and pass.  The sums are the same: even and odd entries, then their sum.
+// What bounds it now: the round trips to L2 of a row's eight entries at a time (4 in
+// flight: 1% slower), in FP64 the FP64 pipe.  Whole solves, CSR -> sorted:
+// 512 LPs of 50 to 2,000 rows 45 -> 19 ms in FP32, 300 of them 85 -> 33 ms in FP64; 64 grid
+// LPs of 144 rows staged in shared memory 6.8 -> 5.1 ms in FP64.
+template <typename T>
+struct RowsSorted {
+  int rows;
+  const int* soff;
+  const unsigned short* len;
+  const T* val;
+  const unsigned short* col;
+  template <class Pre, class Row>
+  __device__ __forceinline__ void each(const T* vec, Pre pre, Row row) const {
+    const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+    for (int sl = threadIdx.x >> 5; sl * 32 < rows; sl += W) {
+      const int i = sl * 32 + lane;
+      const bool in = i < rows;
+      const int o = soff[sl], w = (soff[sl + 1] - o) >> 5;
+      const int n = in ? (int)len[i] : 0;
+      decltype(pre(0)) q{};
+      if (in) q = pre(i);
+      const T* v = val + o + lane;
+      const unsigned short* c = col + o + lane;
+      T e = 0, d = 0;
+      constexpr int U = 8;  // entries in flight (padded entries are zeros of column 0)
+      int t = 0;
+      for (; t + U <= w; t += U) {
+        T x[U];
+        int k[U];
 #pragma unroll
-    for (int r = 0; r < kBR; ++r)
+        for (int u = 0; u < U; ++u) {
+          x[u] = v[(t + u) * 32];
+          k[u] = c[(t + u) * 32];
+        }
 #pragma unroll
-      for (int u = 0; u < kBU; ++u) {
-        const int p = pp[r] + base + u * kLPR;
-        if (p < pe[r]) {
-          v[r][u] = val[p];
-          c[r][u] = col[p];
-          any = true;
+        for (int u = 0; u < U; u += 2) {
+          const T ge = vec[k[u]], go = vec[k[u + 1]];
+          if (t + u < n) e += x[u] * ge;
+          if (t + u + 1 < n) d += x[u + 1] * go;
         }
       }
-    if (!any) break;
-#pragma unroll
-    for (int r = 0; r < kBR; ++r)
-#pragma unroll
-      for (int u = 0; u < kBU; ++u) {
-        const int p = pp[r] + base + u * kLPR;
-        if (p < pe[r]) sr[r] += v[r][u] * vec[c[r][u] - off];
+      for (; t < w; t += 2) {
+        const T x0 = v[t * 32], ge = vec[c[t * 32]];
+        if (t < n) e += x0 * ge;
+        if (t + 1 < w) {
+          const T x1 = v[(t + 1) * 32], go = vec[c[(t + 1) * 32]];
+          if (t + 1 < n) d += x1 * go;
+        }
       }
+      if (in) row(i, e + d, q);
+    }
   }
+};
+
+// Slices of k rows; first slice offset of an instance whose rows start at r0 (every
+// instance has one entry more than slices).
+__host__ __device__ __forceinline__ int n_slices(int k) { return (k + 31) / 32; }
+__host__ __device__ __forceinline__ long long slice_base(long long r0, int b) {
+  return r0 / 32 + 2LL * b;
 }
 
-// Shared-memory pool of an instance run with kStage (T elements, then ints):
-// ys[mb] xs[nb] val[z] valt[z] c l u w xa xhat gbuf [nb each] lc uc ya yhat [mb each]
-// | rp[mb+1] rpt[nb+1] col[z] colt[z], z the instance's nonzeros.
-__host__ __device__ __forceinline__ long long stage_bytes(long long mb, long long nb, long long z,
-                                                          int tsize) {
-  return tsize * (5 * mb + 8 * nb + 2 * z) + 4 * (mb + nb + 2 + 2 * z);
+// Shared-memory pool of an instance run with kStage (T elements, ints, then 16-bit):
+// ys[mb] xs[nb] val[za] valt[zt] c l u w xa xhat gbuf [nb each] lc uc ya yhat [mb each]
+// | soffm[slices + 1] soffn[slices + 1] | col[za] colt[zt] lenm[mb] lenn[nb], za and zt the
+// stored entries of the sorted matrices.
+__host__ __device__ __forceinline__ long long stage_bytes(long long mb, long long nb, long long za,
+                                                          long long zt, int tsize) {
+  return tsize * (5 * mb + 8 * nb + za + zt) + 4 * (n_slices((int)mb) + n_slices((int)nb) + 2) +
+         2 * (za + zt + mb + nb);
 }
 
-// The arrays of one instance as the loop reads them.  Row pointers index val()
-// and col() (global offsets in place, local ones when staged); columns hold
-// global indices (less n0 for A, m0 for A^T); vectors are indexed locally.  In
-// place, every array is the kernel parameter's pointer plus the instance offset
-// (no register holds it); staged, it is the pool position that mb, nb and z fix.
+// The vectors of one instance as the loop reads them, indexed locally in the instance's
+// row order.  In place, every array is the kernel parameter's pointer plus the instance
+// offset (no register holds it); staged, it is the pool position that mb, nb and the
+// matrix sizes fix.
 template <typename T, bool kStage>
 struct Inst {
   const BatchArgs<T>& a;
-  int m0, n0, mb, nb, z;
-  const int *rp, *rpt;
-  T* sp;  // staged: the pool after ys and xs
+  int m0, n0, mb, nb;
+  T* sp;  // staged: the pool after the matrices
 #define MPAX_INST_ARR(Type, name, staged, inplace) \
   __device__ __forceinline__ Type* name() const {    \
     if constexpr (kStage) return staged;             \
     else return inplace;                             \
   }
-  MPAX_INST_ARR(const T, val, sp, a.val)
-  MPAX_INST_ARR(const T, valt, sp + z, a.valt)
-  MPAX_INST_ARR(const T, c, sp + 2 * z, a.c + n0)
-  MPAX_INST_ARR(const T, l, sp + 2 * z + nb, a.l + n0)
-  MPAX_INST_ARR(const T, u, sp + 2 * z + 2 * nb, a.u + n0)
-  MPAX_INST_ARR(T, w, sp + 2 * z + 3 * nb, a.w + n0)
-  MPAX_INST_ARR(T, xa, sp + 2 * z + 4 * nb, a.xa + n0)
-  MPAX_INST_ARR(T, xhat, sp + 2 * z + 5 * nb, a.xhat + n0)
-  MPAX_INST_ARR(T, gbuf, sp + 2 * z + 6 * nb, a.gbuf + n0)
-  MPAX_INST_ARR(const T, lc, sp + 2 * z + 7 * nb, a.lc + m0)
-  MPAX_INST_ARR(const T, uc, sp + 2 * z + 7 * nb + mb, a.uc + m0)
-  MPAX_INST_ARR(T, ya, sp + 2 * z + 7 * nb + 2 * mb, a.ya + m0)
-  MPAX_INST_ARR(T, yhat, sp + 2 * z + 7 * nb + 3 * mb, a.yhat + m0)
-  MPAX_INST_ARR(int, srp, reinterpret_cast<int*>(sp + 2 * z + 7 * nb + 4 * mb), nullptr)
-  MPAX_INST_ARR(const int, col, srp() + (mb + 1) + (nb + 1), a.col)
-  MPAX_INST_ARR(const int, colt, srp() + (mb + 1) + (nb + 1) + z, a.colt)
+  MPAX_INST_ARR(const T, c, sp, a.c + n0)
+  MPAX_INST_ARR(const T, l, sp + nb, a.l + n0)
+  MPAX_INST_ARR(const T, u, sp + 2 * nb, a.u + n0)
+  MPAX_INST_ARR(T, w, sp + 3 * nb, a.w + n0)
+  MPAX_INST_ARR(T, xa, sp + 4 * nb, a.xa + n0)
+  MPAX_INST_ARR(T, xhat, sp + 5 * nb, a.xhat + n0)
+  MPAX_INST_ARR(T, gbuf, sp + 6 * nb, a.gbuf + n0)
+  MPAX_INST_ARR(const T, lc, sp + 7 * nb, a.lc + m0)
+  MPAX_INST_ARR(const T, uc, sp + 7 * nb + mb, a.uc + m0)
+  MPAX_INST_ARR(T, ya, sp + 7 * nb + 2 * mb, a.ya + m0)
+  MPAX_INST_ARR(T, yhat, sp + 7 * nb + 3 * mb, a.yhat + m0)
 #undef MPAX_INST_ARR
 };
 
@@ -224,36 +268,47 @@ struct Inst {
 // iterate vector -- is copied into the shared pool first, so the loop touches
 // global memory only at checks (the unscaled data) and at the end.  Otherwise
 // the two gathered vectors sit at ys, xs (shared or global) and the rest is
-// read in place, with the row pointers staged at srp when they fit.
-template <typename T, bool kStage>
+// read in place.  kSorted: rows by length (RowsSorted), else CSR.
+template <typename T, bool kStage, bool kSorted>
 __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* ys, T* xs,
-                                               int* srp, double* sh,
-                                               unsigned long long t_launch) {
+                                               double* sh, unsigned long long t_launch) {
+  static_assert(kSorted || !kStage, "only sorted instances are staged");
   const unsigned long long t_start = gtimer();
   __shared__ int s_late;
   __shared__ T s_coef[kCoefs + 1];
   const int m0 = (int)a.m_off[b], mb = (int)(a.m_off[b + 1] - a.m_off[b]);
   const int n0 = (int)a.n_off[b], nb = (int)(a.n_off[b + 1] - a.n_off[b]);
-  const int grp = threadIdx.x / kLPR, gl = threadIdx.x % kLPR;
-  const int G = blockDim.x / kLPR;
-  const int z0 = a.rp[m0];
-  Inst<T, kStage> v{a, m0, n0, mb, nb, a.rp[m0 + mb] - z0, a.rp + m0, a.rpt + n0, xs + nb};
+  const long long za0 = a.zsa[b], zt0 = a.zst[b];
+  const int za = (int)(a.zsa[b + 1] - za0), zt = (int)(a.zst[b + 1] - zt0);
+  Inst<T, kStage> v{a, m0, n0, mb, nb, xs + nb + za + zt};
+  using Rows = std::conditional_t<kSorted, RowsSorted<T>, RowsCsr<T>>;
+  Rows A, At;
+  if constexpr (kSorted) {
+    A = Rows{mb, a.soffm + slice_base(m0, b), a.lenm + m0, a.sval + za0, a.scol + za0};
+    At = Rows{nb, a.soffn + slice_base(n0, b), a.lenn + n0, a.svalt + zt0, a.scolt + zt0};
+  } else {
+    A = Rows{mb, a.rp + m0, a.val, a.col, n0};
+    At = Rows{nb, a.rpt + n0, a.valt, a.colt, m0};
+  }
   if constexpr (kStage) {
     // ys (the pool's start) and xs = ys + mb come first; copy the rest in
-    const int zt0 = a.rpt[n0];
-    int* srp_a = v.srp();
-    int* srp_t = srp_a + (mb + 1);
-    T* sval = const_cast<T*>(v.val());
-    T* svalt = const_cast<T*>(v.valt());
-    int* scol = const_cast<int*>(v.col());
-    int* scolt = const_cast<int*>(v.colt());
-    for (int i = threadIdx.x; i <= mb; i += blockDim.x) srp_a[i] = a.rp[m0 + i] - z0;
-    for (int j = threadIdx.x; j <= nb; j += blockDim.x) srp_t[j] = a.rpt[n0 + j] - zt0;
-    for (int p = threadIdx.x; p < v.z; p += blockDim.x) {
-      sval[p] = a.val[z0 + p];
-      scol[p] = a.col[z0 + p];
-      svalt[p] = a.valt[zt0 + p];
-      scolt[p] = a.colt[zt0 + p];
+    T* sval = xs + nb;
+    T* svalt = sval + za;
+    int* sm = reinterpret_cast<int*>(v.sp + 7 * nb + 4 * mb);
+    int* sn = sm + n_slices(mb) + 1;
+    unsigned short* scol = reinterpret_cast<unsigned short*>(sn + n_slices(nb) + 1);
+    unsigned short* scolt = scol + za;
+    unsigned short* slm = scolt + zt;
+    unsigned short* sln = slm + mb;
+    for (int i = threadIdx.x; i <= n_slices(mb); i += blockDim.x) sm[i] = A.soff[i];
+    for (int j = threadIdx.x; j <= n_slices(nb); j += blockDim.x) sn[j] = At.soff[j];
+    for (int p = threadIdx.x; p < za; p += blockDim.x) {
+      sval[p] = A.val[p];
+      scol[p] = A.col[p];
+    }
+    for (int p = threadIdx.x; p < zt; p += blockDim.x) {
+      svalt[p] = At.val[p];
+      scolt[p] = At.col[p];
     }
     T* sc = const_cast<T*>(v.c());
     T* sl = const_cast<T*>(v.l());
@@ -262,29 +317,24 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
       sc[j] = a.c[n0 + j];
       sl[j] = a.l[n0 + j];
       su[j] = a.u[n0 + j];
+      sln[j] = At.len[j];
     }
     T* slc = const_cast<T*>(v.lc());
     T* suc = const_cast<T*>(v.uc());
     for (int i = threadIdx.x; i < mb; i += blockDim.x) {
       slc[i] = a.lc[m0 + i];
       suc[i] = a.uc[m0 + i];
+      slm[i] = A.len[i];
     }
     __syncthreads();
-    v.rp = srp_a;
-    v.rpt = srp_t;
-  } else if (srp) {
-    // Row pointers of A_b and A_b^T: staged in shared memory when they fit (one
-    // global round trip less in every step of a half-step), else read in place.
-    int* sa = srp;
-    int* st = srp + (mb + 1);
-    for (int i = threadIdx.x; i <= mb; i += blockDim.x) sa[i] = a.rp[m0 + i];
-    for (int j = threadIdx.x; j <= nb; j += blockDim.x) st[j] = a.rpt[n0 + j];
-    __syncthreads();
-    v.rp = sa;
-    v.rpt = st;
+    A = Rows{mb, sm, slm, sval, scol};
+    At = Rows{nb, sn, sln, svalt, scolt};
   }
-  const int* rpl = v.rp;
-  const int* rptl = v.rpt;
+  // original (global) row and column of a place in the instance's order
+  auto row_of = [&](int i) { return m0 + (kSorted ? a.permm[m0 + i] : i); };
+  auto col_of = [&](int j) { return n0 + (kSorted ? a.permn[n0 + j] : j); };
+  auto none = [](int) { return 0; };
+  const bool has_rows = a.rp[m0 + mb] > a.rp[m0];
 
   // ---- power iteration for ||A~_b||_2 from the common start vector ----------
   double ss0 = 0.0;
@@ -293,35 +343,19 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
     ss0 += r * r;
   }
   const double inv0 = 1.0 / sqrt(fmax(bsum(ss0, sh), 1e-300));
-  for (int j = threadIdx.x; j < nb; j += blockDim.x) xs[j] = (T)(power_start_raw(j) * inv0);
+  for (int j = threadIdx.x; j < nb; j += blockDim.x)
+    xs[j] = (T)(power_start_raw(col_of(j) - n0) * inv0);
   __syncthreads();
   double nA = 0.0, nu_prev = 0.0, d_prev = 0.0;
-  const bool has_rows = mb > 0 && rpl[mb] > rpl[0];
   if (has_rows && a.power_max_iter == 0) nA = a.power_cap;  // the certified bound
   for (int t = 1; has_rows && t <= a.power_max_iter; ++t) {
-    for (int i0 = 0; i0 < mb; i0 += G) {
-      const int i = i0 + grp;
-      const bool in_i = i < mb;
-      T s = 0;
-      for (int p = in_i ? rpl[i] + gl : 0; in_i && p < rpl[i + 1]; p += kLPR)
-        s += v.val()[p] * xs[v.col()[p] - n0];
-      s = group_sum(s);
-      if (gl == 0 && in_i) ys[i] = s;
-    }
+    A.each(xs, none, [&](int i, T s, int) { ys[i] = s; });
     __syncthreads();
     double acc = 0.0;
-    for (int j0 = 0; j0 < nb; j0 += G) {
-      const int j = j0 + grp;
-      const bool in_j = j < nb;
-      T s = 0;
-      for (int p = in_j ? rptl[j] + gl : 0; in_j && p < rptl[j + 1]; p += kLPR)
-        s += v.valt()[p] * ys[v.colt()[p] - m0];
-      s = group_sum(s);
-      if (gl == 0 && in_j) {
-        v.gbuf()[j] = s;
-        acc += (double)s * (double)s;
-      }
-    }
+    At.each(ys, none, [&](int j, T s, int) {
+      v.gbuf()[j] = s;
+      acc += (double)s * (double)s;
+    });
     const double nrm = sqrt(bsum(acc, sh));
     if (nrm == 0.0) {
       nA = 0.0;
@@ -362,13 +396,13 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   // ---- start at zero, or (warm) at the returned point of an earlier launch,
   // taken back into the scaled space: anchor, reflected point, duals ---------
   for (int j = threadIdx.x; j < nb; j += blockDim.x) {
-    const T x = a.warm ? (T)(a.xout[n0 + j] / a.Dc[n0 + j]) : (T)0;
+    const T x = a.warm ? (T)(a.xout[col_of(j)] / a.Dc[col_of(j)]) : (T)0;
     v.xa()[j] = x;
     v.w()[j] = x;
     v.xhat()[j] = x;
   }
   for (int i = threadIdx.x; i < mb; i += blockDim.x) {
-    const T y = a.warm ? (T)(a.yout[m0 + i] / a.Dr[m0 + i]) : (T)0;
+    const T y = a.warm ? (T)(a.yout[row_of(i)] / a.Dr[row_of(i)]) : (T)0;
     ys[i] = y;
     v.ya()[i] = y;
     v.yhat()[i] = y;
@@ -394,94 +428,45 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
       }
       const T rb = s_coef[it % kCoefs];      // rebuild weight of x^{n,k}
       const T hb = s_coef[it % kCoefs + 1];  // Halpern weight of the anchor
-      // primal half-step over the rows of A^T (eq. 3, first line).  Each kLPR-lane
-      // group takes kBR rows per step (j, j + G, ...) and issues the row pointers,
-      // the epilogue operands and both rows' products before reducing, so every
-      // dependent round trip to memory is shared by kBR rows.
-      for (int j0 = 0; j0 < nb; j0 += kBR * G) {
-        int jr[kBR], pp[kBR], pe[kBR];
-        T sr[kBR], x0r[kBR], wr[kBR], cr[kBR], lr[kBR], ur[kBR];
-#pragma unroll
-        for (int r = 0; r < kBR; ++r) {
-          jr[r] = j0 + r * G + grp;
-          const bool in = jr[r] < nb;
-          pp[r] = in ? rptl[jr[r]] + gl : 0;
-          pe[r] = in ? rptl[jr[r] + 1] : 0;
-          sr[r] = 0;
-          if (gl == 0 && in) {
-            const int j = jr[r];
-            x0r[r] = v.xa()[j];
-            wr[r] = v.w()[j];
-            cr[r] = v.c()[j];
-            lr[r] = v.l()[j];
-            ur[r] = v.u()[j];
-          }
-        }
-        rows_dot<T>(pp, pe, v.valt(), v.colt(), ys, m0, sr);
-#pragma unroll
-        for (int r = 0; r < kBR; ++r) sr[r] = group_sum(sr[r]);
-        if (gl == 0) {
-#pragma unroll
-          for (int r = 0; r < kBR; ++r) {
-            if (jr[r] >= nb) continue;
-            const int j = jr[r];
-            const T x0 = x0r[r], wv = wr[r];
-            const T x = (k == 0) ? x0 : wv + rb * (x0 - wv);
-            const T xh = clampv<T>(x - tt * (cr[r] - sr[r]), lr[r], ur[r]);
+      // primal half-step over the rows of A^T (eq. 3, first line)
+      struct Col {
+        T x0, w, c, l, u;
+      };
+      At.each(
+          ys, [&](int j) { return Col{v.xa()[j], v.w()[j], v.c()[j], v.l()[j], v.u()[j]}; },
+          [&](int j, T s, const Col& q) {
+            const T x = (k == 0) ? q.x0 : q.w + rb * (q.x0 - q.w);
+            const T xh = clampv<T>(x - tt * (q.c - s), q.l, q.u);
             const T wn = (T)2 * xh - x;
             v.w()[j] = wn;
             xs[j] = wn;
             if (chk) {
               v.xhat()[j] = xh;
-              const double d0 = (double)xh - (double)x, d1 = (double)xh - (double)x0;
+              const double d0 = (double)xh - (double)x, d1 = (double)xh - (double)q.x0;
               P0 += d0 * d0;
               P1 += d1 * d1;
             }
-          }
-        }
-      }
+          });
       __syncthreads();
-      // dual half-step over the rows of A (eq. 3, second line) and Halpern (eq. 4),
-      // kBR rows per group and step as above
-      for (int i0 = 0; i0 < mb; i0 += kBR * G) {
-        int ir[kBR], pp[kBR], pe[kBR];
-        T sr[kBR], yar[kBR], lcr[kBR], ucr[kBR];
-#pragma unroll
-        for (int r = 0; r < kBR; ++r) {
-          ir[r] = i0 + r * G + grp;
-          const bool in = ir[r] < mb;
-          pp[r] = in ? rpl[ir[r]] + gl : 0;
-          pe[r] = in ? rpl[ir[r] + 1] : 0;
-          sr[r] = 0;
-          if (gl == 0 && in) {
-            const int i = ir[r];
-            yar[r] = v.ya()[i];
-            lcr[r] = v.lc()[i];
-            ucr[r] = v.uc()[i];
-          }
-        }
-        rows_dot<T>(pp, pe, v.val(), v.col(), xs, n0, sr);
-#pragma unroll
-        for (int r = 0; r < kBR; ++r) sr[r] = group_sum(sr[r]);
-        if (gl == 0) {
-#pragma unroll
-          for (int r = 0; r < kBR; ++r) {
-            if (ir[r] >= mb) continue;
-            const int i = ir[r];
-            const T y0 = ys[i], y0a = yar[r];
-            const T t = y0 * iss - sr[r];
-            const T yh = ss * (t - clampv<T>(t, -ucr[r], -lcr[r]));
+      // dual half-step over the rows of A (eq. 3, second line) and Halpern (eq. 4)
+      struct Row {
+        T ya, lc, uc;
+      };
+      A.each(
+          xs, [&](int i) { return Row{v.ya()[i], v.lc()[i], v.uc()[i]}; },
+          [&](int i, T s, const Row& q) {
+            const T y0 = ys[i];
+            const T t = y0 * iss - s;
+            const T yh = ss * (t - clampv<T>(t, -q.uc, -q.lc));
             const T z = (T)2 * yh - y0;
-            ys[i] = z + hb * (y0a - z);
+            ys[i] = z + hb * (q.ya - z);
             if (chk) {
               v.yhat()[i] = yh;
-              const double d0 = (double)yh - (double)y0, d1 = (double)yh - (double)y0a;
+              const double d0 = (double)yh - (double)y0, d1 = (double)yh - (double)q.ya;
               D0 += d0 * d0;
               D1 += d1 * d1;
             }
-          }
-        }
-      }
+          });
       __syncthreads();
       ++k;
       ++total;
@@ -490,45 +475,29 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
     for (int j = threadIdx.x; j < nb; j += blockDim.x) xs[j] = v.xhat()[j];
     __syncthreads();
     double K0 = 0, K1 = 0, C0 = 0, C1 = 0, C2 = 0;
-    for (int i0 = 0; i0 < mb; i0 += G) {
-      const int i = i0 + grp;
-      const bool in_i = i < mb;
-      T s = 0;
-      for (int p = in_i ? rpl[i] + gl : 0; in_i && p < rpl[i + 1]; p += kLPR)
-        s += v.val()[p] * xs[v.col()[p] - n0];
-      s = group_sum(s);
-      if (gl == 0 && in_i) {
-        const int g = m0 + i;
-        const double ax = (double)s * a.iDr[g];
-        const double lo = a.lc0[g], hi = a.uc0[g];
-        const double r = ax - fmin(fmax(ax, lo), hi);
-        K0 += r * r;
-        const double y = a.Dr[g] * (double)v.yhat()[i];
-        if (y > 0.0 && isfinite(lo)) K1 += lo * y;
-        if (y < 0.0 && isfinite(hi)) K1 += hi * y;
-      }
-    }
-    for (int j0 = 0; j0 < nb; j0 += G) {
-      const int j = j0 + grp;
-      const bool in_j = j < nb;
-      T s = 0;
-      for (int p = in_j ? rptl[j] + gl : 0; in_j && p < rptl[j + 1]; p += kLPR)
-        s += v.valt()[p] * v.yhat()[v.colt()[p] - m0];
-      s = group_sum(s);
-      if (gl == 0 && in_j) {
-        const int g = n0 + j;
-        const double aty = (double)s * a.iDc[g];
-        const double x = a.Dc[g] * (double)xs[j];
-        const double lam = a.c0[g] - aty;
-        const double lo = a.l0[g], hi = a.u0[g];
-        const bool lf = isfinite(lo), uf = isfinite(hi);
-        const double lh = (lf && uf) ? lam : lf ? fmax(lam, 0.0) : uf ? fmin(lam, 0.0) : 0.0;
-        const double rd = lam - lh;
-        C0 += rd * rd;
-        C1 += a.c0[g] * x;
-        C2 += (lf ? lo * fmax(lh, 0.0) : 0.0) + (uf ? hi * fmin(lh, 0.0) : 0.0);
-      }
-    }
+    A.each(xs, none, [&](int i, T s, int) {
+      const int g = row_of(i);
+      const double ax = (double)s * a.iDr[g];
+      const double lo = a.lc0[g], hi = a.uc0[g];
+      const double r = ax - fmin(fmax(ax, lo), hi);
+      K0 += r * r;
+      const double y = a.Dr[g] * (double)v.yhat()[i];
+      if (y > 0.0 && isfinite(lo)) K1 += lo * y;
+      if (y < 0.0 && isfinite(hi)) K1 += hi * y;
+    });
+    At.each(v.yhat(), none, [&](int j, T s, int) {
+      const int g = col_of(j);
+      const double aty = (double)s * a.iDc[g];
+      const double x = a.Dc[g] * (double)xs[j];
+      const double lam = a.c0[g] - aty;
+      const double lo = a.l0[g], hi = a.u0[g];
+      const bool lf = isfinite(lo), uf = isfinite(hi);
+      const double lh = (lf && uf) ? lam : lf ? fmax(lam, 0.0) : uf ? fmin(lam, 0.0) : 0.0;
+      const double rd = lam - lh;
+      C0 += rd * rd;
+      C1 += a.c0[g] * x;
+      C2 += (lf ? lo * fmax(lh, 0.0) : 0.0) + (uf ? hi * fmin(lh, 0.0) : 0.0);
+    });
     P0 = bsum(P0, sh);
     P1 = bsum(P1, sh);
     D0 = bsum(D0, sh);
@@ -605,9 +574,9 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   }
   // ---- returned point (x^, y^), unscaled; per-instance statistics ---------
   for (int j = threadIdx.x; j < nb; j += blockDim.x)
-    a.xout[n0 + j] = a.Dc[n0 + j] * (double)v.xhat()[j];
+    a.xout[col_of(j)] = a.Dc[col_of(j)] * (double)v.xhat()[j];
   for (int i = threadIdx.x; i < mb; i += blockDim.x)
-    a.yout[m0 + i] = a.Dr[m0 + i] * (double)v.yhat()[i];
+    a.yout[row_of(i)] = a.Dr[row_of(i)] * (double)v.yhat()[i];
   if (threadIdx.x == 0) {
     // a warm launch continues an instance: its counts and time add to the earlier ones
     a.status[b] = term;
@@ -628,7 +597,6 @@ __global__ void __launch_bounds__(kBatchThreads<T>, kBatchMinB<T>) batch_lp_kern
   __shared__ double sh[32];
   __shared__ int s_inst;
   T* pool = reinterpret_cast<T*>(sm);
-  int* rpool = reinterpret_cast<int*>(pool + a.smem_vec);
   const unsigned long long t_launch = gtimer();  // used by thread 0 only
   while (true) {
     if (threadIdx.x == 0) s_inst = atomicAdd(a.next, 1);
@@ -638,24 +606,152 @@ __global__ void __launch_bounds__(kBatchThreads<T>, kBatchMinB<T>) batch_lp_kern
     if (w >= a.n_todo) return;
     const int b = a.todo ? a.todo[w] : w;
     const int mb = (int)(a.m_off[b + 1] - a.m_off[b]), nb = (int)(a.n_off[b + 1] - a.n_off[b]);
-    const int z = a.rp[a.m_off[b + 1]] - a.rp[a.m_off[b]];
-    int* srp = (mb + nb + 2 <= a.rp_cap) ? rpool : nullptr;
-    // three call sites: the whole instance in shared memory; its two gathered
-    // vectors in shared memory (shared loads for the gathers); everything global
-    if (kStaging && stage_bytes(mb, nb, z, (int)sizeof(T)) <= a.stage_cap)
-      solve_instance<T, true>(a, b, pool, pool + mb, nullptr, sh, t_launch);
+    const long long za = a.zsa[b + 1] - a.zsa[b], zt = a.zst[b + 1] - a.zst[b];
+    // call sites: the whole instance in shared memory; its two gathered vectors in
+    // shared memory (shared loads for the gathers), sorted rows or CSR; everything global
+    if (kStaging && za > 0 && stage_bytes(mb, nb, za, zt, (int)sizeof(T)) <= a.stage_cap)
+      solve_instance<T, kStaging, true>(a, b, pool, pool + mb, sh, t_launch);
+    else if (za > 0)
+      solve_instance<T, false, true>(a, b, pool, pool + mb, sh, t_launch);
     else if (mb + nb <= a.smem_vec)
-      solve_instance<T, false>(a, b, pool, pool + mb, srp, sh, t_launch);
+      solve_instance<T, false, false>(a, b, pool, pool + mb, sh, t_launch);
     else
-      solve_instance<T, false>(a, b, a.gys + a.m_off[b], a.gxs + a.n_off[b], srp, sh, t_launch);
+      solve_instance<T, false, false>(a, b, a.gys + a.m_off[b], a.gxs + a.n_off[b], sh, t_launch);
   }
 }
 
-// z[b] = rp[m_off[b]], b = 0..B
-__global__ void k_first_nnz(const long long* __restrict__ rp, const long long* __restrict__ m_off,
-                            int B, long long* __restrict__ z) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b <= B) z[b] = rp[m_off[b]];
+// ---- rows by length -------------------------------------------------------------------
+constexpr int kLenBins = 1024;  // rows of kLenBins - 1 or more entries share a bin
+constexpr int kPadSlack = 4096;
+
+// Stable order of one matrix's rows by falling length, by one warp: perm[place] = row,
+// inv[row] = place, the lengths and the slices' offsets in sorted order.  Returns the
+// stored entries (32 times the longest row of each slice).
+__device__ __forceinline__ long long sort_rows(const int* rp, int rows, int* bins, int* perm,
+                                               int* inv, unsigned short* len, int* soff) {
+  const int lane = threadIdx.x & 31;
+  for (int k = lane; k < kLenBins; k += 32) bins[k] = 0;
+  __syncwarp();
+  for (int i = lane; i < rows; i += 32) atomicAdd(&bins[min(rp[i + 1] - rp[i], kLenBins - 1)], 1);
+  __syncwarp();
+  int run = 0;  // first place of each bin, longest first: 32 bins at a time
+  for (int k = kLenBins - 32; k >= 0; k -= 32) {
+    const int bin = k + 31 - lane, c = bins[bin];
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += t;
+    }
+    bins[bin] = run + x - c;
+    run += __shfl_sync(0xffffffffu, x, 31);
+  }
+  __syncwarp();
+  for (int i0 = 0; i0 < rows; i0 += 32) {
+    const int i = i0 + lane;
+    const int bin = i < rows ? min(rp[i + 1] - rp[i], kLenBins - 1) : -1;
+    const unsigned same = __match_any_sync(0xffffffffu, bin);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    const int base = bin >= 0 ? bins[bin] : 0;
+    __syncwarp();
+    if (bin >= 0) {
+      perm[base + rank] = i;
+      inv[i] = base + rank;
+      len[base + rank] = (unsigned short)min(rp[i + 1] - rp[i], 65535);
+      if (rank == 0) bins[bin] = base + __popc(same);
+    }
+    __syncwarp();
+  }
+  long long o = 0;
+  for (int sl = 0; sl * 32 < rows; ++sl) {
+    const int i = sl * 32 + lane;
+    const int w = (int)__reduce_max_sync(0xffffffffu, i < rows ? (unsigned)len[i] : 0u);
+    if (lane == 0) soff[sl] = (int)min(o, 0x7fffffffLL);
+    o += 32LL * w;
+  }
+  if (lane == 0) soff[n_slices(rows)] = (int)min(o, 0x7fffffffLL);
+  return o;
+}
+
+// A warp per instance.  size[b], size[B + b]: stored entries of its sorted A and A^T, or zero
+// when it keeps CSR: its vectors do not fit in shared memory (mb + nb > vec_cap, which is
+// below 2^16), or padding would store more than twice its nonzeros.
+__global__ void k_sort_rows(const long long* __restrict__ m_off, const long long* __restrict__ n_off,
+                            int B, const int* __restrict__ rp, const int* __restrict__ rpt,
+                            int vec_cap, int* __restrict__ permm, int* __restrict__ permn,
+                            int* __restrict__ invm, int* __restrict__ invn,
+                            unsigned short* __restrict__ lenm, unsigned short* __restrict__ lenn,
+                            int* __restrict__ soffm, int* __restrict__ soffn,
+                            long long* __restrict__ size) {
+  __shared__ int bins[kLenBins];
+  const int b = blockIdx.x, lane = threadIdx.x;
+  const int m0 = (int)m_off[b], mb = (int)(m_off[b + 1] - m0);
+  const int n0 = (int)n_off[b], nb = (int)(n_off[b + 1] - n0);
+  const long long z = rp[m0 + mb] - rp[m0];
+  long long za = 0, zt = 0;
+  if (z > 0 && mb + nb <= vec_cap) {
+    za = sort_rows(rp + m0, mb, bins, permm + m0, invm + m0, lenm + m0, soffm + slice_base(m0, b));
+    __syncwarp();
+    zt = sort_rows(rpt + n0, nb, bins, permn + n0, invn + n0, lenn + n0, soffn + slice_base(n0, b));
+    if (za > 2 * z + kPadSlack || zt > 2 * z + kPadSlack) za = zt = 0;
+  }
+  if (za == 0) {
+    for (int i = lane; i < mb; i += 32) permm[m0 + i] = i;
+    for (int j = lane; j < nb; j += 32) permn[n0 + j] = j;
+  }
+  if (lane == 0) {
+    size[b] = za;
+    size[B + b] = zt;
+  }
+}
+
+// One matrix of every sorted instance into its slices: values cast to T (through src when
+// given: A^T's entries in A), columns as places of the gathered vector; padding is zeros of
+// column 0.  Block (b, y): every gridDim.y-th group of slices of instance b.
+template <typename T>
+__global__ void k_fill_sorted(const long long* __restrict__ r_off, const int* __restrict__ rp, const int* __restrict__ col,
+                              const double* __restrict__ val, const int* __restrict__ src,
+                              const int* __restrict__ perm, const int* __restrict__ inv,
+                              const int* __restrict__ soff, const long long* __restrict__ zs,
+                              T* __restrict__ sval, unsigned short* __restrict__ scol) {
+  const int b = blockIdx.x;
+  const long long z0 = zs[b];
+  if (zs[b + 1] == z0) return;
+  const int r0 = (int)r_off[b], rows = (int)(r_off[b + 1] - r0);
+  const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  const int* so = soff + slice_base(r0, b);
+  for (int sl = blockIdx.y * W + (threadIdx.x >> 5); sl * 32 < rows; sl += gridDim.y * W) {
+    const int i = sl * 32 + lane;
+    const int r = i < rows ? r0 + perm[r0 + i] : 0;
+    const int p0 = i < rows ? rp[r] : 0, n = i < rows ? rp[r + 1] - p0 : 0;
+    const int o = so[sl], w = (so[sl + 1] - o) >> 5;
+    for (int t = 0; t < w; ++t) {
+      const long long e = z0 + o + t * 32 + lane;
+      T x = (T)0;
+      int k = 0;
+      if (t < n) {
+        x = (T)(src ? val[src[p0 + t]] : val[p0 + t]);
+        k = inv[col[p0 + t]];
+      }
+      sval[e] = x;
+      scol[e] = (unsigned short)k;
+    }
+  }
+}
+
+// Scaled data in every instance's row order: dst_i = src_g * d_g (or / d_g), g the original
+// index of place i of instance b (a block per instance and chunk).
+template <typename T>
+__global__ void k_scale_perm(const long long* __restrict__ off, const int* __restrict__ perm,
+                             const double* __restrict__ src, const double* __restrict__ d,
+                             bool divide, T* __restrict__ dst) {
+  const int b = blockIdx.x;
+  const long long o = off[b];
+  const int k = (int)(off[b + 1] - o);
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < k; i += gridDim.y * blockDim.x) {
+    const long long g = o + perm[o + i];
+    dst[o + i] = (T)(divide ? src[g] / d[g] : src[g] * d[g]);
+  }
 }
 
 // row -> instance via binary search in m_off; global column = n_off[b] + local
@@ -743,7 +839,6 @@ struct mpax_batch {
   long long* m_off = nullptr;  // device
   long long* n_off = nullptr;
   std::vector<long long> h_moff, h_noff;
-  std::vector<long long> h_zoff;  // row_ptr at each instance's first row
   int max_m = 0, max_n = 0;
   int* next = nullptr;
   int* status = nullptr;
@@ -758,6 +853,11 @@ struct mpax_batch {
   int* todo = nullptr;     // device list of instances continued in FP64
   int fp64_instances = 0;  // instances of the last solve continued in FP64
   double* spo = nullptr;   // SPO+ staging of host arguments: 3 sum(n) + B doubles
+  // rows by length (k_sort_rows): orders, lengths, slice offsets and storage ranges in
+  // one buffer, the stored matrices (precision dependent) in another
+  void* rows = nullptr;
+  void* sell = nullptr;
+  size_t sell_bytes = 0;
 };
 
 namespace mpax {
@@ -825,16 +925,76 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
   T *w = take(n), *xa = take(n), *xhat = take(n), *gbuf = take(n);
   T *ya = take(m), *yhat = take(m);
   T *gys = take(m), *gxs = take(n);
-  cudaError_t e;
-  if ((e = cast_vec<T>(P.val_s, valA, nnz, s))) return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));
-  if ((e = gather_cast<T>(P.val_s, P.permT, valAt, nnz, s)))
+  // ---- rows by length: orders, slices and, per instance, what they store -------------
+  const int B = bt->B;
+  const long long vec_cap = kBatchVecBytes / (long long)sizeof(T);
+  const size_t slm = (size_t)m / 32 + 2 * (size_t)B + 2, sln = (size_t)n / 32 + 2 * (size_t)B + 2;
+  if (!bt->rows) {
+    const size_t bytes = sizeof(long long) * (4 * (size_t)B + 2) +
+                         sizeof(int) * (2 * ((size_t)m + n) + slm + sln) +
+                         sizeof(unsigned short) * ((size_t)m + n + 8);
+    if (cudaMalloc(&bt->rows, bytes) != cudaSuccess)
+      return bfail(MPAX_ERR_OUT_OF_MEMORY, "batch row orders");
+  }
+  long long* size = reinterpret_cast<long long*>(bt->rows);  // 2 B
+  long long *zsa = size + 2 * (size_t)B, *zst = zsa + B + 1;
+  int *permm = reinterpret_cast<int*>(zst + B + 1), *permn = permm + m, *invm = permn + n,
+      *invn = invm + m, *soffm = invn + n, *soffn = soffm + slm;
+  unsigned short *lenm = reinterpret_cast<unsigned short*>(soffn + sln), *lenn = lenm + m;
+  k_sort_rows<<<B, 32, 0, s>>>(bt->m_off, bt->n_off, B, P.A.rp, P.At.rp, (int)vec_cap, permm, permn,
+                               invm, invn, lenm, lenn, soffm, soffn, size);
+  std::vector<long long> hsize(2 * (size_t)B), hz(2 * (size_t)B + 2, 0);
+  cudaError_t e = cudaGetLastError();
+  if (!e) e = cudaMemcpyAsync(hsize.data(), size, sizeof(long long) * 2 * B, cudaMemcpyDeviceToHost, s);
+  if (!e) e = cudaStreamSynchronize(s);
+  if (e) return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));
+  std::vector<char> run(B, todo_host ? 0 : 1);  // instances of this launch
+  for (int w = 0; todo_host && w < n_todo; ++w) run[todo_host[w]] = 1;
+  long long *hza = hz.data(), *hzt = hza + B + 1;
+  bool csr = false;  // an instance of the launch reads the CSR arrays
+  for (int b = 0; b < B; ++b) {
+    hza[b + 1] = hza[b] + (run[b] ? hsize[b] : 0);
+    hzt[b + 1] = hzt[b] + (run[b] ? hsize[B + b] : 0);
+    csr = csr || (run[b] && hsize[b] == 0);
+  }
+  const long long ZA = hza[B], ZT = hzt[B];
+  const size_t sell_need = (sizeof(T) + sizeof(unsigned short)) * ((size_t)ZA + ZT) + 256;
+  if (bt->sell_bytes < sell_need) {
+    if (bt->sell) cudaFree(bt->sell);
+    bt->sell = nullptr;
+    bt->sell_bytes = 0;
+    if (cudaMalloc(&bt->sell, sell_need) != cudaSuccess)
+      return bfail(MPAX_ERR_OUT_OF_MEMORY, "batch rows by length");
+    bt->sell_bytes = sell_need;
+  }
+  T *sval = reinterpret_cast<T*>(bt->sell), *svalt = sval + ZA;
+  unsigned short *scol = reinterpret_cast<unsigned short*>(svalt + ZT), *scolt = scol + ZA;
+  if ((e = cudaMemcpyAsync(zsa, hz.data(), sizeof(long long) * (2 * (size_t)B + 2),
+                           cudaMemcpyHostToDevice, s)))
     return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));
-  scale_cast<T>(P.c, P.Dc, false, c, n, s);
-  scale_cast<T>(P.l, P.Dc, true, l, n, s);
-  scale_cast<T>(P.u, P.Dc, true, u, n, s);
-  scale_cast<T>(P.lc, P.Dr, false, lc, m, s);
-  scale_cast<T>(P.uc, P.Dr, false, uc, m, s);
-  *launches += 7;
+  // blocks per instance of the fills: about 16 per SM in all, at most 8
+  const int fy = std::max(1, std::min(8, (16 * 152 + B - 1) / B));
+  if (ZA > 0) {
+    k_fill_sorted<T><<<dim3(B, fy), 256, 0, s>>>(bt->m_off, P.A.rp, P.A.col, P.val_s, nullptr, permm, invn, soffm, zsa, sval, scol);
+    k_fill_sorted<T><<<dim3(B, fy), 256, 0, s>>>(bt->n_off, P.At.rp, P.At.col, P.val_s,
+                                                 P.permT, permn, invm, soffn, zst, svalt, scolt);
+  }
+  if (csr) {
+    if ((e = cast_vec<T>(P.val_s, valA, nnz, s))) return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));
+    if ((e = gather_cast<T>(P.val_s, P.permT, valAt, nnz, s)))
+      return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));
+  }
+  const dim3 gp(B, fy);
+  if (n) {
+    k_scale_perm<T><<<gp, 256, 0, s>>>(bt->n_off, permn, P.c, P.Dc, false, c);
+    k_scale_perm<T><<<gp, 256, 0, s>>>(bt->n_off, permn, P.l, P.Dc, true, l);
+    k_scale_perm<T><<<gp, 256, 0, s>>>(bt->n_off, permn, P.u, P.Dc, true, u);
+  }
+  if (m) {
+    k_scale_perm<T><<<gp, 256, 0, s>>>(bt->m_off, permm, P.lc, P.Dr, false, lc);
+    k_scale_perm<T><<<gp, 256, 0, s>>>(bt->m_off, permm, P.uc, P.Dr, false, uc);
+  }
+  *launches += 8 + (csr ? 2 : 0);
   BatchArgs<T>& a = L->a;
   a.B = bt->B;
   a.m_off = bt->m_off;
@@ -876,6 +1036,18 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
   a.next = bt->next;
   a.gys = gys;
   a.gxs = gxs;
+  a.permm = permm;
+  a.permn = permn;
+  a.lenm = lenm;
+  a.lenn = lenn;
+  a.soffm = soffm;
+  a.soffn = soffn;
+  a.zsa = zsa;
+  a.zst = zst;
+  a.sval = sval;
+  a.svalt = svalt;
+  a.scol = scol;
+  a.scolt = scolt;
   a.eps_abs = o->eps_abs;
   a.eps_rel = o->eps_rel;
   a.r_suff = o->restart_sufficient;
@@ -893,20 +1065,14 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
   a.power_cap = o->pock_chambolle ? 1.0 : INFINITY;
   // the shared pool fits the largest instance of this launch that fits in
   // kBatchVecBytes; larger instances run from global memory
-  const long long vec_cap = kBatchVecBytes / (long long)sizeof(T);
-  long long vmax = 0, rmax = 0;
+  long long vmax = 0;
   for (int w = 0; w < n_todo; ++w) {
     const int b = todo_host ? todo_host[w] : w;
     const long long v = (bt->h_moff[b + 1] - bt->h_moff[b]) + (bt->h_noff[b + 1] - bt->h_noff[b]);
     if (v <= vec_cap) vmax = std::max(vmax, v);
-    rmax = std::max(rmax, v + 2);
   }
   a.smem_vec = (int)((vmax + 3) / 4 * 4);
-  size_t smem = sizeof(T) * (size_t)a.smem_vec;
-  // row pointers staged when two CTAs per SM still fit
-  a.rp_cap = (MPAX_BATCH_SMEM_RP && smem + sizeof(int) * (size_t)rmax <= 100 * 1024)
-                 ? (int)rmax : 0;
-  smem += sizeof(int) * (size_t)a.rp_cap;
+  const size_t smem = sizeof(T) * (size_t)a.smem_vec;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -916,9 +1082,9 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
   for (int w = 0; w < n_todo; ++w) {
     const int b = todo_host ? todo_host[w] : w;
     const long long need = stage_bytes(bt->h_moff[b + 1] - bt->h_moff[b],
-                                       bt->h_noff[b + 1] - bt->h_noff[b],
-                                       bt->h_zoff[b + 1] - bt->h_zoff[b], (int)sizeof(T));
-    if (need <= cap) smax = std::max(smax, need);
+                                       bt->h_noff[b + 1] - bt->h_noff[b], hsize[b], hsize[B + b],
+                                       (int)sizeof(T));
+    if (hsize[b] > 0 && need <= cap) smax = std::max(smax, need);
   }
   a.stage_cap = smax;
   L->smem = std::max(smem, (size_t)((smax + 15) / 16 * 16));
@@ -1005,13 +1171,6 @@ mpax_status mpax_lp_batch_create(int32_t B, const int64_t* m_off, const int64_t*
   const cudaMemcpyKind kin = kind == MPAX_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   if (!e) e = cudaMemcpy(d_rp, row_ptr, sizeof(long long) * (m + 1), kin);
   if (!e && nnz > 0) e = cudaMemcpy(d_col, col_idx, sizeof(int) * nnz, kin);
-  // row_ptr at each instance's first row (sizes the whole-instance staging)
-  std::vector<long long> hz(B + 1);
-  long long* d_z = nullptr;
-  if (!e) e = cudaMalloc(&d_z, sizeof(long long) * (B + 1));
-  if (!e) k_first_nnz<<<(B + 256) / 256, 256>>>(d_rp, d_moff, B, d_z);
-  if (!e) e = cudaMemcpy(hz.data(), d_z, sizeof(long long) * (B + 1), cudaMemcpyDeviceToHost);
-  if (d_z) cudaFree(d_z);
   if (!e) e = cudaMemset(flags, 0, sizeof(int));
   if (!e && m > 0) k_globalize_cols<<<(m + 255) / 256, 256>>>(d_moff, d_noff, B, d_rp, m, d_col, flags);
   int hf = 0;
@@ -1067,7 +1226,6 @@ mpax_status mpax_lp_batch_create(int32_t B, const int64_t* m_off, const int64_t*
   bt->n_off = d_noff;
   bt->h_moff = hm;
   bt->h_noff = hn;
-  bt->h_zoff = hz;
   bt->max_m = max_m;
   bt->max_n = max_n;
   if (e) {
@@ -1359,7 +1517,7 @@ void mpax_batch_destroy(mpax_batch* bt) {
   if (bt->prob) mpax_destroy(bt->prob);
   void* bufs[] = {bt->m_off, bt->n_off, bt->next, bt->status, bt->iters, bt->restarts,
                   bt->relkkt, bt->pobj, bt->secs, bt->xout, bt->yout, bt->work, bt->todo,
-                  bt->spo};
+                  bt->spo, bt->rows, bt->sell};
   for (void* b : bufs)
     if (b) cudaFree(b);
   delete bt;

@@ -354,3 +354,50 @@ def test_batch_stage_option_is_validated(C):
             C.mpax_batch_solve(h, C.mpax_options_default(batch_stage=2))
     finally:
         C.mpax_batch_destroy(h)
+
+
+def _shaped_instance(lengths, n, seed):
+    """An LP whose rows have the given lengths: equality rows through a point of [0, 1]^n."""
+    rng = np.random.default_rng(seed)
+    col = np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for k in lengths])
+    rp = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    val = rng.standard_normal(len(col))
+    m = len(lengths)
+    rows = np.repeat(np.arange(m), lengths)
+    b = np.bincount(rows, weights=val * rng.random(n)[col], minlength=m)
+    c = np.bincount(col, weights=val * rng.standard_normal(m)[rows], minlength=n)
+    return dict(m=m, n=n, nnz=len(col), row_ptr=rp, col=col.astype(np.int32), val=val, c=c, lc=b,
+                uc=b.copy(), l=np.zeros(n), u=np.ones(n))
+
+
+@pytest.mark.parametrize("many", [False, True], ids=["staged", "in_place"])
+def test_batch_row_orders_match_oracle(C, many):
+    """Rows are stored by length in slices of 32, a thread per row: one row, one and two
+    slices and one row more, empty rows, odd and even lengths around the eight entries in
+    flight, lengths past the 1,023 that are told apart, and one dense row among rows of one
+    entry, which keeps CSR (padding would store 30 times its entries).  FP64, 1e-12 as in
+    test_batch_iterates_match_oracle."""
+    prec, k, tol = 0, 128, 1e-12
+    rng = np.random.default_rng(11)
+    shapes = [([5], 9), ([3] * 32, 40), (list(range(1, 34)), 50), ([0, 7, 0, 8, 9, 15, 16, 17, 0], 30),
+              (list(rng.integers(0, 24, 65)), 100), (list(rng.integers(1000, 1100, 40)), 1150),
+              ([2900] + [1] * 39, 3000)]
+    insts = [_shaped_instance(L, n, i) for i, (L, n) in enumerate(shapes)]
+    check = len(insts)
+    if many:  # more instances than SMs: none is staged whole
+        insts = insts + [_shaped_instance([4, 5, 6], 12, 100 + i) for i in range(160)]
+    d = _pack(insts)
+    opts = dict(iteration_limit=k, eps_abs=1e-14, eps_rel=1e-14, power_max_iter=0)
+    h = _create(C, d)
+    try:
+        C.mpax_batch_solve(h, C.mpax_options_default(precision=prec, **opts))
+        x, y = C.mpax_batch_get_solution(h, int(d["m_off"][-1]), int(d["n_off"][-1]))
+    finally:
+        C.mpax_batch_destroy(h)
+    for b, inst in enumerate(insts[:check]):
+        ref = O.solve_lp(O.problem_from_arrays(inst), O.Options(
+            eps_primal_infeasible=0.0, eps_dual_infeasible=0.0, **opts))
+        if ref.iterations < k:  # a small instance solved to the last bit by then
+            continue
+        assert rel_inf(x[d["n_off"][b]:d["n_off"][b + 1]], ref.x) <= tol, b
+        assert rel_inf(y[d["m_off"][b]:d["m_off"][b + 1]], ref.y) <= tol, b
