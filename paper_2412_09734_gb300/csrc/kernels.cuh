@@ -40,12 +40,15 @@ struct SpmvArgs {
   int q0;        // first partial slot used by this launch
 };
 
-// Input gathers.
-template <typename T>
+// Input gathers.  kShared: the vector changes while the kernel runs (power.cuh), so it is
+// read through L2; otherwise through the read-only path.
+template <typename T, bool kShared = false>
 struct InPlain {
   const T* x;
   __device__ __forceinline__ void load() {}
-  __device__ __forceinline__ T operator()(int j) const { return ld_ro(x + j); }
+  __device__ __forceinline__ T operator()(int j) const {
+    return kShared ? __ldcg(x + j) : ld_ro(x + j);
+  }
 };
 
 // x_md = xavg + beta (x - xavg), beta = coef_a[it] (rAPDHG momentum point, eq. 6)
@@ -63,6 +66,12 @@ struct InMomentum {
   }
 };
 
+// Matrix values and columns: kept in L1, or streamed past it.
+template <bool kResident, typename V>
+__device__ __forceinline__ V ld_matrix(const V* p) {
+  return kResident ? __ldg(p) : ld_stream(p);
+}
+
 __device__ __forceinline__ int item_row(const int4& it) { return it.x >= 0 ? it.x : -(it.x + 1); }
 
 __device__ __forceinline__ void item_range(const int4& it, int& p0, int& p1) {
@@ -73,21 +82,6 @@ __device__ __forceinline__ void item_range(const int4& it, int& p0, int& p1) {
     p0 = it.y;
     p1 = it.z;
   }
-}
-
-// Programmatic dependent launch (sm_90+ griddepcontrol).  launch_dependents lets
-// the next kernel of the stream start its CTAs once every CTA of this grid has
-// issued it or exited; wait returns when the previous grid has completed and its
-// memory operations are visible.  Without the launch attribute both are no-ops.
-__device__ __forceinline__ void pdl_launch_dependents() {
-#if MPAX_SPMV_PDL
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-#endif
-}
-__device__ __forceinline__ void pdl_wait() {
-#if MPAX_SPMV_PDL
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-#endif
 }
 
 // TMA bulk prefetch of [p, p + bytes) into L2 (16-byte aligned, rounded out;
@@ -203,18 +197,13 @@ constexpr int kSpmvBufLen = kFmaRows<T> ? 2 * kShortCap + (kRowWords * 4 + 7) / 
 template <typename T>
 using SpmvBuf = T[kSpmvWarps][kSpmvBufLen<T>];
 
-// The work of CTA `cta` of a spmv_fused launch over the items of `a`: one item
-// per warp.
-template <typename T, class In, class Epi>
-__device__ __forceinline__ void spmv_fused_cta(const SpmvArgs<T>& a, In& in, Epi& epi, int cta,
-                                               SpmvBuf<T>& sbuf) {
+// One item by one warp; buf: the warp's kSpmvBufLen<T> elements of shared memory.
+// kResident: a kernel that walks the same items again and again (power.cuh) keeps the
+// matrix in L1; otherwise it streams past L1.
+template <typename T, class In, class Epi, bool kResident = false>
+__device__ __forceinline__ void spmv_item(const SpmvArgs<T>& a, In& in, Epi& epi, int item,
+                                          T* buf) {
   const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  const int item = cta * kSpmvWarps + wib;
-  // The next launch may start its CTAs as this grid drains (programmatic
-  // dependent launch); it reads only the constant matrix arrays before its wait.
-  pdl_launch_dependents();
-  if (item >= a.n_items) return;
   const int4 it = a.items[item];
   const bool do_pf = (lane == 0) && a.pf_dist > 0 && item + a.pf_dist < a.n_items;
 
@@ -232,14 +221,12 @@ __device__ __forceinline__ void spmv_fused_cta(const SpmvArgs<T>& a, In& in, Epi
     for (int u = 0; u < kShortLoads; ++u) {
       const int q = base + lane + u * kWarp;
       if (q < end) {
-        v[u] = ld_stream(a.val + q);
-        c[u] = ld_stream(a.col + q);
+        v[u] = ld_matrix<kResident>(a.val + q);
+        c[u] = ld_matrix<kResident>(a.col + q);
       }
     }
     int4 ft;
     if (do_pf) ft = a.items[item + a.pf_dist];
-    // everything below reads or writes state of the previous launches
-    pdl_wait();
     if (epi.skip()) return;
     in.load();
     epi.load();
@@ -249,7 +236,6 @@ __device__ __forceinline__ void spmv_fused_cta(const SpmvArgs<T>& a, In& in, Epi
     typename Epi::Pre pra, prb;
     epi.pre(sa, pra);
     epi.pre(sb, prb);
-    T* buf = sbuf[wib];
     T* bufx = buf + kShortCap;  // FP64 only: the gathered inputs
 #pragma unroll
     for (int u = 0; u < kShortLoads; ++u) {
@@ -300,13 +286,12 @@ __device__ __forceinline__ void spmv_fused_cta(const SpmvArgs<T>& a, In& in, Epi
   for (int u = 0; u < kSliceLoads; ++u) {
     const int q = p0 + lane + u * kWarp;
     if (q < p1) {
-      v[u] = ld_stream(a.val + q);
-      c[u] = ld_stream(a.col + q);
+      v[u] = ld_matrix<kResident>(a.val + q);
+      c[u] = ld_matrix<kResident>(a.col + q);
     }
   }
   int4 ft;
   if (do_pf) ft = a.items[item + a.pf_dist];
-  pdl_wait();
   if (epi.skip()) return;
   in.load();
   epi.load();
@@ -374,6 +359,16 @@ __device__ __forceinline__ void spmv_fused_cta(const SpmvArgs<T>& a, In& in, Epi
       }
     }
   }
+}
+
+// The work of CTA `cta` of a spmv_fused launch over the items of `a`: one item
+// per warp.
+template <typename T, class In, class Epi>
+__device__ __forceinline__ void spmv_fused_cta(const SpmvArgs<T>& a, In& in, Epi& epi, int cta,
+                                               SpmvBuf<T>& sbuf) {
+  const int wib = threadIdx.x >> 5;
+  const int item = cta * kSpmvWarps + wib;
+  if (item < a.n_items) spmv_item<T, In, Epi>(a, in, epi, item, sbuf[wib]);
 }
 
 // MINB: resident CTAs per SM asked of the register allocator (the default

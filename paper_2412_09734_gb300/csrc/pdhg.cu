@@ -20,6 +20,7 @@
 #include "engine.cuh"
 #include "epilogues.cuh"
 #include "kernels.cuh"
+#include "power.cuh"
 #include "spmv_launch.cuh"
 #include "unrolled.cuh"
 
@@ -664,9 +665,15 @@ class Engine final : public EngineBase {
       }
     }
     st_ = dalloc<DevState>(1, e);
+    bar_.w = dalloc<unsigned>(kGridBarWords, e);
+    csum_ = dalloc<double>(kRoundMaxCtas, e);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev);
     if (*e == cudaSuccess) *e = cudaHostAlloc(&hs_, sizeof(HostStatus), cudaHostAllocMapped);
     if (*e == cudaSuccess) *e = cudaHostGetDevicePointer((void**)&hs_dev_, hs_, 0);
     if (*e == cudaSuccess) *e = cudaMemsetAsync(st_, 0, sizeof(DevState), P->s);
+    if (*e == cudaSuccess) *e = cudaMemsetAsync(bar_.w, 0, sizeof(unsigned) * kGridBarWords, P->s);
   }
 
   ~Engine() override {
@@ -675,7 +682,7 @@ class Engine final : public EngineBase {
     void* bufs[] = {valA_, valAt_, c_,    l_,    u_,    lc_,   uc_,    xbar_, wbuf_,
                     xa_,   xhat_,  xprev_, pv_,  pg_,   y_,    ya_,    yhat_, yprev_,
                     pw_,   x_,     xavg_, xref_, xanc_, yavg_, yanc_,  Ds_,   fval_,
-                    ftval_, uvec_, uvec2_, rayx_, rayy_, qv_, qvec_, qvec2_, st_};
+                    ftval_, uvec_, uvec2_, rayx_, rayy_, qv_, qvec_, qvec2_, st_, bar_.w, csum_};
     for (void* b : bufs)
       if (b) cudaFree(b);
     if (hs_) cudaFreeHost(hs_);
@@ -735,6 +742,34 @@ class Engine final : public EngineBase {
     T* v = pv_;
     T* g = pg_;
     const int* skip = &st_->pw_done;
+    // all rounds in one launch where the products are small (power.cuh); a caller that
+    // names a kernel of the products gets it
+    if (o.spmv_kernel < 0) {
+      const bool two = mode == 0 || !P.q_general;
+      SpmvArgs<T> a1{}, a2{};
+      if (mode == 0) {
+        a1 = fused_args<T>(P.schedA, P.A, valA_, 0);
+        a2 = fused_args<T>(P.schedAt, P.At, valAt_, 0);
+      } else if (P.q_general) {
+        a2 = fused_args<T>(P.schedQ, P.Q, qv_, 0);
+      } else {
+        a1 = fused_args<T>(P.schedFt, P.Ft, ftval_, 0);
+        a2 = fused_args<T>(P.schedF, P.F, fval_, 0);
+      }
+      const int most = std::max(a1.n_items, a2.n_items);
+      if (a2.n_items > 0 && round_fits(most, sms_)) {
+        const double cap = mode == 0 && o.pock_chambolle ? 1.0 : INFINITY;
+        const cudaError_t e = launch_cooperative(
+            power_rounds<T>, round_ctas(most, sms_), 32 * kRoundWarps, kRoundSmem<T>, s, a1, a2,
+            (int)two, v, g, mode == 0 ? pw_ : uvec_, mode == 1 && two ? (const T*)Ds_ : nullptr,
+            (int)(mode == 0), o.power_tol, cap, (int)o.power_max_iter, csum_, st_, bar_);
+        if (!e) {
+          *launches += 1;
+          return barrier_error();
+        }
+        cudaGetLastError();  // not all CTAs fit at once (a partitioned GPU): launched rounds
+      }
+    }
     for (int t = 1; t <= o.power_max_iter; ++t) {
       EpiStore<T> e1{skip, nullptr, &st_->pw_scale, nullptr, nullptr, nullptr, 0};
       EpiStore<T> e2{skip, g, nullptr, nullptr, nullptr, nullptr, 1};
@@ -851,6 +886,15 @@ class Engine final : public EngineBase {
       if (h) return cudaErrorTimeout;
     }
     return cudaSuccess;
+  }
+  // A barrier of power_rounds that gave up: cudaErrorTimeout, and the words are zeroed.
+  cudaError_t barrier_error() {
+    unsigned b = 0;
+    cudaError_t e = cudaMemcpyAsync(&b, bar_.w + 2, sizeof(b), cudaMemcpyDeviceToHost, P_->s);
+    if (!e) e = cudaStreamSynchronize(P_->s);
+    if (e || !b) return e;
+    if ((e = cudaMemsetAsync(bar_.w, 0, sizeof(unsigned) * kGridBarWords, P_->s))) return e;
+    return cudaErrorTimeout;
   }
 
   // One launch of the iteration's half-step on schedule q (0: A, the dual step;
@@ -1593,6 +1637,9 @@ class Engine final : public EngineBase {
   T *yavg_ = nullptr, *yanc_ = nullptr;
   T *Ds_ = nullptr, *fval_ = nullptr, *ftval_ = nullptr, *uvec_ = nullptr, *uvec2_ = nullptr;
   T *qv_ = nullptr, *qvec_ = nullptr, *qvec2_ = nullptr;  // general sparse Q
+  GridBar bar_{nullptr};     // barrier and chunk sums of power_rounds
+  double* csum_ = nullptr;
+  int sms_ = 1;
   DevState* st_ = nullptr;
   HostStatus* hs_ = nullptr;
   HostStatus* hs_dev_ = nullptr;

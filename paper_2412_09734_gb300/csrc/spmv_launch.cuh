@@ -94,21 +94,7 @@ void launch_spmv(const Sched& sc, const Csr& K, const T* val, In in, Epi epi, in
     spmv_fused<T, In, Epi, kSpmvWideMinB><<<grid, kSpmvBlock, 0, s>>>(a, in, epi);
     return;
   }
-#if MPAX_SPMV_PDL
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kSpmvBlock);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, spmv_fused<T, In, Epi>, a, in, epi);
-#else
   spmv_fused<T, In, Epi><<<grid, kSpmvBlock, 0, s>>>(a, in, epi);
-#endif
 }
 
 // The arguments of a spmv_fused launch over schedule sc (no prefetch).
