@@ -293,14 +293,17 @@ __global__ void k_power_finalize(const double* __restrict__ part, int n, DevStat
   }
 }
 
-__device__ double sum_slot(const double* part, int q, int n, double* sh) {
+// Sum of n values by one warp, lane i adding values i, i + 32, ... (valid in lane 0).
+__device__ __forceinline__ double warp_slot_sum(const double* __restrict__ p, int n) {
   double v = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v += part[(size_t)q * n + i];
-  return block_sum(v, sh);
+  for (int i = threadIdx.x & 31; i < n; i += 32) v += p[i];
+  return warp_sum(v);
 }
 
 // First level of the check reductions: block b sums the fixed chunk b of every
-// partial-sum slot (A^T slots 0..qt-1, then A slots 0..qa-1) into out[q][b].
+// partial-sum slot (A^T slots 0..qt-1, then A slots 0..qa-1) into out[q][b], a warp per
+// slot.  One after another over the whole block, the sixteen slots of a check took two
+// block barriers each, here and in the finalizer (34 -> 12 us, on one CTA).
 constexpr int kChunks = 128;
 // Check quantities reduced per check: 10 partial slots of the A^T schedule
 // (0-1 restart metric, 2-5 KKT columns, 6-9 ray columns) then 6 of the A
@@ -309,17 +312,14 @@ constexpr int kCheckQt = 10, kCheckQa = 6, kCheckQ = kCheckQt + kCheckQa;
 __global__ void k_part_reduce(const double* __restrict__ partAt, int nAt, int qt,
                               const double* __restrict__ partA, int nA, int qa,
                               const int* skip, double* __restrict__ out) {
-  __shared__ double sh[32];
   if (skip && *skip) return;
-  for (int q = 0; q < qt + qa; ++q) {
+  for (int q = threadIdx.x >> 5; q < qt + qa; q += blockDim.x >> 5) {
     const double* p = q < qt ? partAt + (size_t)q * nAt : partA + (size_t)(q - qt) * nA;
     const int n = q < qt ? nAt : nA;
     const int chunk = (n + kChunks - 1) / kChunks;
     const int lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
-    double v = 0;
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) v += p[i];
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) out[q * kChunks + blockIdx.x] = v;
+    const double v = warp_slot_sum(p + lo, max(0, hi - lo));
+    if ((threadIdx.x & 31) == 0) out[q * kChunks + blockIdx.x] = v;
   }
 }
 
@@ -329,13 +329,12 @@ __global__ void k_part_reduce(const double* __restrict__ partAt, int nAt, int qt
 __global__ void k_finalize_check(const double* __restrict__ partAt, int nAt,
                                  const double* __restrict__ partA, int nA, DevState* st,
                                  HostStatus* hs, int len, int next_len) {
-  __shared__ double sh[32];
   __shared__ double vals[kCheckQ];
   if (st->done) return;
   // partAt / partA hold the kChunks first-level sums of every slot (k_part_reduce)
-  for (int q = 0; q < kCheckQ; ++q) {
-    const double v = sum_slot(partAt, q, kChunks, sh);
-    if (threadIdx.x == 0) vals[q] = v;
+  for (int q = threadIdx.x >> 5; q < kCheckQ; q += blockDim.x >> 5) {
+    const double v = warp_slot_sum(partAt + (size_t)q * kChunks, kChunks);
+    if ((threadIdx.x & 31) == 0) vals[q] = v;
   }
   (void)partA;
   (void)nA;
@@ -491,17 +490,12 @@ __global__ void k_restart_qp(const DevState* st, int n, int m, const T* __restri
 __global__ void k_kkt_finalize(const double* __restrict__ partAt, int nAt,
                                const double* __restrict__ partA, int nA, const DevState* st,
                                double* out) {
-  __shared__ double sh[32];
   __shared__ double vals[6];
   // partAt holds the chunk sums of the A^T slots 0..kCheckQt-1 then the A slots
   // (KKT columns in A^T slots 2..5, KKT rows in A slots 2..3)
-  for (int q = 0; q < 4; ++q) {
-    const double v = sum_slot(partAt, 2 + q, nAt, sh);
-    if (threadIdx.x == 0) vals[q] = v;
-  }
-  for (int q = 0; q < 2; ++q) {
-    const double v = sum_slot(partAt, kCheckQt + 2 + q, nAt, sh);
-    if (threadIdx.x == 0) vals[4 + q] = v;
+  for (int q = threadIdx.x >> 5; q < 6; q += blockDim.x >> 5) {
+    const double v = warp_slot_sum(partAt + (size_t)(2 + (q < 4 ? q : kCheckQt + q - 4)) * nAt, nAt);
+    if ((threadIdx.x & 31) == 0) vals[q] = v;
   }
   (void)partA;
   (void)nA;
@@ -1056,7 +1050,7 @@ class Engine final : public EngineBase {
     if (plain) return;
     kkt_launch(&st_->done, prof);
     if (!qp) ray_launch(&st_->done);
-    k_part_reduce<<<kChunks, 256, 0, s>>>(P.schedAt.part, P.schedAt.n_items, kCheckQt,
+    k_part_reduce<<<kChunks, 512, 0, s>>>(P.schedAt.part, P.schedAt.n_items, kCheckQt,
                                           P.schedA.part, P.schedA.n_items, kCheckQa,
                                           &st_->done, P.red);
     k_finalize_check<<<1, 512, 0, s>>>(P.red, kChunks, nullptr, 0, st_, hs_dev_, len, block_);
@@ -1612,7 +1606,7 @@ class Engine final : public EngineBase {
     if (P.schedA.part) cudaMemsetAsync(P.schedA.part, 0, sizeof(double) * kPartQ * std::max(P.schedA.n_items, 1), s);
     if (P.schedAt.part) cudaMemsetAsync(P.schedAt.part, 0, sizeof(double) * kPartQ * std::max(P.schedAt.n_items, 1), s);
     kkt_launch(nullptr, false);
-    k_part_reduce<<<kChunks, 256, 0, s>>>(P.schedAt.part, P.schedAt.n_items, kCheckQt,
+    k_part_reduce<<<kChunks, 512, 0, s>>>(P.schedAt.part, P.schedAt.n_items, kCheckQt,
                                           P.schedA.part, P.schedA.n_items, 4, nullptr, P.red);
     k_kkt_finalize<<<1, 256, 0, s>>>(P.red, kChunks, nullptr, 0, st_, out6);
     return cudaGetLastError();
