@@ -357,13 +357,25 @@ __global__ void k_coefs(const Inst* __restrict__ inst, int B, int it0, int len,
 }
 
 // The sum of `chunks` partial vectors of length len at coordinate e, in order (B = 1:
-// the matrix-vector product's partials); the loads of eight chunks are in flight at once.
+// the matrix-vector product's partials), the loads of kPartsAhead chunks in flight at once.
+// One instance has too few coordinates to hide them otherwise: 1000 x 100,000, primal
+// and dual update 7.6 and 6.0 us with eight, 6.2 and 4.6 us with sixteen.
+constexpr int kPartsAhead = 16;
 template <int V>
 __device__ __forceinline__ void sum_parts(const float* part, int chunks, int len, int e, float* t) {
 #pragma unroll
   for (int i = 0; i < V; ++i) t[i] = 0.0f;
-#pragma unroll 8
-  for (int c = 0; c < chunks; ++c) {
+  int c = 0;
+  for (; c + kPartsAhead <= chunks; c += kPartsAhead) {
+    float q[kPartsAhead][V];
+#pragma unroll
+    for (int u = 0; u < kPartsAhead; ++u) ld_vec<V>(part, (size_t)(c + u) * len + e, q[u]);
+#pragma unroll
+    for (int u = 0; u < kPartsAhead; ++u)
+#pragma unroll
+      for (int i = 0; i < V; ++i) t[i] += q[u][i];
+  }
+  for (; c < chunks; ++c) {
     float q[V];
     ld_vec<V>(part, (size_t)c * len + e, q);
 #pragma unroll
