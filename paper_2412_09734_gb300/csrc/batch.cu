@@ -27,13 +27,19 @@
 
 namespace mpax {
 
-// Threads of the CTA that solves one instance, one CTA per SM.  FP32: 1024 at 64 registers
-// (2,000 instances of 50 to 2,000 rows 56 ms; two CTAs of 512 71 ms); FP64: 512 at 128
-// registers (300 of them 33 ms; two CTAs of 512 at 64 registers, which spill, 40 ms).
+// Threads of the CTA that solves one instance.  FP64: 512 at 128 registers, one CTA per SM
+// (300 instances of 50 to 2,000 rows 33 ms; two CTAs of 512 at 64 registers, which spill,
+// 40 ms).  FP32: one CTA of 1024 at 64 registers, or two of 512 where there are more
+// instances than such CTAs and they are small, at most kSmallCols columns on average and
+// kSmallVec rows and columns each: their slices of 32 rows leave many of 32 warps idle.
+// Measured, 1024 / 2 x 512 threads: 2,000 instances of 320 columns on average 13.2 / 8.6 ms,
+// 1,500 of 850 12.9 / 10.2, 1,000 of 1,200 12.3 / 10.5, 2,000 of 2,050 56 / 71; 100 of 620
+// 3.2 / 3.7.
 template <typename T>
 constexpr int kBatchThreads = sizeof(T) == 4 ? 1024 : 512;
-template <typename T>
-constexpr int kBatchMinB = 1;
+constexpr int kBatchSmallThreads = 512;
+constexpr int kSmallCols = 1400;
+constexpr int kSmallVec = 25000;  // rows + columns: the vectors of two CTAs fit in one SM
 constexpr double kBatchMaxSeconds = 600.0;
 // Partial sums of a row: entries 0, 2, 4, ... and 1, 3, 5, ..., added at the end.  In CSR
 // (RowsCsr) two lanes hold them.  Rows of the batch recipe hold ~1-40 nonzeros: measured on 4096 instances, 2 lanes per
@@ -591,8 +597,9 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
 
 // kStaging: the launch may stage whole instances (a separate instantiation, so
 // that the many-instance kernel carries only the two in-place call sites).
-template <typename T, bool kStaging>
-__global__ void __launch_bounds__(kBatchThreads<T>, kBatchMinB<T>) batch_lp_kernel(BatchArgs<T> a) {
+template <typename T, bool kStaging, int kThreads>
+__global__ void __launch_bounds__(kThreads, kBatchThreads<T> / kThreads)
+    batch_lp_kernel(BatchArgs<T> a) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ double sh[32];
   __shared__ int s_inst;
@@ -1116,10 +1123,26 @@ mpax_status run_batch(mpax_batch* bt, const mpax_options* o, long long* launches
                                     true, &bt->work, &bt->work_bytes, &L);
   if (st) return st;
   cudaStream_t s = problem_data(bt->prob)->s;
-  auto kernel = L.a.stage_cap > 0 ? batch_lp_kernel<T, true> : batch_lp_kernel<T, false>;
-  const int grid = batch_grid(kernel, kBatchThreads<T>, L.smem, n_todo);
+  constexpr int kT = kBatchThreads<T>;
+  auto kernel = L.a.stage_cap > 0 ? batch_lp_kernel<T, true, kT> : batch_lp_kernel<T, false, kT>;
+  int threads = kT;
+  if constexpr (kT > kBatchSmallThreads) {
+    // by the batch's sizes alone, so that staging or not stays the same bits
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    bool small = bt->B > 2 * sms && bt->h_noff[bt->B] <= (long long)kSmallCols * bt->B;
+    for (int b = 0; b < bt->B && small; ++b)
+      small = bt->h_moff[b + 1] - bt->h_moff[b] + bt->h_noff[b + 1] - bt->h_noff[b] <= kSmallVec;
+    if (small) {
+      kernel = L.a.stage_cap > 0 ? batch_lp_kernel<T, true, kBatchSmallThreads>
+                                 : batch_lp_kernel<T, false, kBatchSmallThreads>;
+      threads = kBatchSmallThreads;
+    }
+  }
+  const int grid = batch_grid(kernel, threads, L.smem, n_todo);
   cudaMemsetAsync(bt->next, 0, sizeof(int), s);
-  kernel<<<grid, kBatchThreads<T>, L.smem, s>>>(L.a);
+  kernel<<<grid, threads, L.smem, s>>>(L.a);
   *launches += 1;
   cudaError_t e = cudaGetLastError();
   if (e) return bfail(MPAX_ERR_CUDA, cudaGetErrorString(e));

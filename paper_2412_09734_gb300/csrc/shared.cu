@@ -14,10 +14,9 @@
 // A_lo X_lo term is of order 2^-16 relative, so a product is accurate to about
 // 2^-16 relative per term (an FP32 product: 2^-24).  The split of
 // the iterates is written by the fused update kernels, so a GEMM reads BF16
-// operands only.  The GEMMs are plain library GEMMs (cuBLAS); the PDHG update,
+// operands only.  The products are the kernels of umma.cuh; the PDHG update,
 // projection, Halpern step, splitting and the FP64 check reductions are this
-// file's kernels.  A plain FP32 product path (SGEMM on the FP32 pipes) is kept
-// for comparison.
+// file's kernels.  The plain FP32 products (sgemm.cuh) run on the FP32 pipes.
 //
 // Layout: A is row-major m x n, i.e. column-major n x m; X, Y and every
 // per-instance vector are column-major (column k = instance k).

@@ -401,3 +401,24 @@ def test_batch_row_orders_match_oracle(C, many):
             continue
         assert rel_inf(x[d["n_off"][b]:d["n_off"][b + 1]], ref.x) <= tol, b
         assert rel_inf(y[d["m_off"][b]:d["m_off"][b + 1]], ref.y) <= tol, b
+
+
+@pytest.mark.parametrize("B", [304, 305, 400])
+def test_batch_small_instances_two_per_sm(C, B):
+    """FP32 batches of many small instances run two CTAs of 512 threads per SM (from 305
+    instances on 152 SMs); every instance meets its tolerance in the oracle's evaluation, on
+    both sides of the line."""
+    d = ragged_lp_batch(B, seed=31, m_lo=20, m_hi=60, density=0.1)
+    h = _create(C, d)
+    try:
+        C.mpax_batch_solve(h, C.mpax_options_default(precision=1, power_max_iter=0,
+                                                     iteration_limit=200000))
+        _, per = C.mpax_batch_get_stats(h, B)
+        x, y = C.mpax_batch_get_solution(h, int(d["m_off"][-1]), int(d["n_off"][-1]))
+    finally:
+        C.mpax_batch_destroy(h)
+    assert np.all(per["status"] == 1)
+    for b in range(0, B, 37):
+        chk = O.kkt(O.problem_from_arrays(d["instances"][b]), x[d["n_off"][b]:d["n_off"][b + 1]],
+                    y[d["m_off"][b]:d["m_off"][b + 1]], 1.5e-4, 1.5e-4)
+        assert chk["converged"], b
