@@ -811,10 +811,10 @@ def run_batch(args):
         ms = e0.elapsed_time(e1) / steps
         summ, per = C.mpax_batch_get_stats(h, d["B"])
         C.mpax_batch_destroy(h)
-        # two matrix passes per iteration over each instance's CSR (values + columns)
+        # two matrix passes per iteration over each instance (values + 16-bit columns)
         vbytes = 4 if name == "mixed" else 8
         nnz_b = np.diff(d["nnz_off"]).astype(np.float64)
-        mat_bytes = float(np.sum(per["iterations"] * 2.0 * nnz_b * (vbytes + 4)))
+        mat_bytes = float(np.sum(per["iterations"] * 2.0 * nnz_b * (vbytes + 2)))
         pk, pk_src = peaks()
         ach = mat_bytes / (ms / 1e3) / 1e9
         out[name] = dict(solves_per_s=d["B"] / (ms / 1e3), ms_per_batch=ms,
