@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "../../include/mpax.h"
+#include "batch_work.h"
 #include "problem.cuh"
 
 namespace mpax {
@@ -911,8 +912,8 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
   cudaStream_t s = P.s;
   const int m = P.m, n = P.n, nnz = P.nnz;
   // scaled data and iterate storage in the iteration precision
-  const size_t need =
-      sizeof(T) * ((size_t)2 * (nnz + kPad) + 10 * (size_t)n + 8 * (size_t)m + 96);
+  const BatchWork at((size_t)m, (size_t)n, (size_t)nnz + kPad);
+  const size_t need = sizeof(T) * at.total;
   if (*work_bytes < need) {
     if (*work) cudaFree(*work);
     *work = nullptr;
@@ -921,17 +922,10 @@ mpax_status batch_prepare(mpax_batch* bt, const mpax_options* o, long long* laun
     *work_bytes = need;
   }
   T* p = reinterpret_cast<T*>(*work);
-  auto take = [&](size_t k) {
-    T* r = p;
-    p += (k + 15) / 16 * 16;
-    return r;
-  };
-  T* valA = take(nnz + kPad);
-  T* valAt = take(nnz + kPad);
-  T *c = take(n), *l = take(n), *u = take(n), *lc = take(m), *uc = take(m);
-  T *w = take(n), *xa = take(n), *xhat = take(n), *gbuf = take(n);
-  T *ya = take(m), *yhat = take(m);
-  T *gys = take(m), *gxs = take(n);
+  T *valA = p + at.val, *valAt = p + at.valt;
+  T *c = p + at.c, *l = p + at.l, *u = p + at.u, *lc = p + at.lc, *uc = p + at.uc;
+  T *w = p + at.w, *xa = p + at.xa, *xhat = p + at.xhat, *gbuf = p + at.gbuf;
+  T *ya = p + at.ya, *yhat = p + at.yhat, *gys = p + at.gys, *gxs = p + at.gxs;
   // ---- rows by length: orders, slices and, per instance, what they store -------------
   const int B = bt->B;
   const long long vec_cap = kBatchVecBytes / (long long)sizeof(T);

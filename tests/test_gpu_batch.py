@@ -422,3 +422,26 @@ def test_batch_small_instances_two_per_sm(C, B):
         chk = O.kkt(O.problem_from_arrays(d["instances"][b]), x[d["n_off"][b]:d["n_off"][b + 1]],
                     y[d["m_off"][b]:d["m_off"][b + 1]], 1.5e-4, 1.5e-4)
         assert chk["converged"], b
+
+
+@pytest.mark.parametrize("prec,eps", [(0, 1e-8), (1, 1e-4)])
+@pytest.mark.parametrize("stage", [0, 1])
+@pytest.mark.parametrize("lengths,n", [([1], 1), ([3], 5), ([0], 4)],
+                         ids=["1x1", "1x5", "no_nonzeros"])
+def test_batch_of_one_tiny_instance(C, lengths, n, stage, prec, eps):
+    """A batch of a handful of rows and columns, whose arrays are shorter than the rounding
+    of their places in the work buffer (test_host_rules.py checks those), in place and staged."""
+    inst = _shaped_instance(lengths, n, 5)
+    inst["c"] = np.random.default_rng(6).standard_normal(n)
+    d = _pack([inst])
+    h = _create(C, d)
+    try:
+        for _ in range(2):  # the second solve finds the buffers of the first
+            C.mpax_batch_solve(h, C.mpax_options_default(precision=prec, eps_abs=eps, eps_rel=eps,
+                                                         batch_stage=stage, iteration_limit=200000))
+            _, per = C.mpax_batch_get_stats(h, 1)
+            x, y = C.mpax_batch_get_solution(h, len(lengths), n)
+            assert per["status"][0] == 1
+            assert O.kkt(O.problem_from_arrays(inst), x, y, 1.5 * eps, 1.5 * eps)["converged"]
+    finally:
+        C.mpax_batch_destroy(h)

@@ -1,0 +1,48 @@
+"""Layouts and predicates that the kernels share with plain C++: compiled with the host
+compiler and checked exhaustively over small values, without a GPU."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2412_09734_gb300", "csrc")
+
+
+@pytest.fixture
+def run_cpp(tmp_path):
+    """Compiles a program against the kernel sources' headers; returns its output's lines."""
+    def go(source):
+        src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
+        src.write_text(source)
+        subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+        return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split("\n")
+    return go
+
+
+def test_batch_work_arrays_stay_apart_and_inside_the_buffer(run_cpp):
+    lines = run_cpp(r"""
+#include <cstdio>
+#include "batch_work.h"
+int main() {
+  for (size_t m = 0; m < 40; m += 1 + m / 3)
+    for (size_t n = 0; n < 150; n += 1 + n / 4)
+      for (size_t za = 16; za < 90; za += 1 + (za - 16) / 2) {
+        mpax::BatchWork w(m, n, za);
+        std::printf("%zu %zu %zu %zu", m, n, za, w.total);
+        const size_t at[15][2] = {{w.val, za}, {w.valt, za}, {w.c, n}, {w.l, n}, {w.u, n},
+                                  {w.lc, m}, {w.uc, m}, {w.w, n}, {w.xa, n}, {w.xhat, n},
+                                  {w.gbuf, n}, {w.ya, m}, {w.yhat, m}, {w.gys, m}, {w.gxs, n}};
+        for (auto& a : at) std::printf(" %zu %zu", a[0], a[1]);
+        std::printf("\n");
+      }
+}
+""")
+    rows = [[int(v) for v in line.split()] for line in lines if line]
+    assert len(rows) > 1000
+    for m, n, za, total, *at in rows:
+        end = 0
+        for start, length in sorted(zip(at[::2], at[1::2])):
+            assert start % 16 == 0 and start >= end, (m, n, za)
+            end = start + length
+        assert end <= total, (m, n, za)
