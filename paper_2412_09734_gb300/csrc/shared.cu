@@ -36,6 +36,7 @@
 #include "../../include/mpax.h"
 #include "umma_host.h"
 #include "common.cuh"
+#include "rules.h"
 #include "sgemm.cuh"
 
 namespace mpax {
@@ -791,12 +792,12 @@ __global__ void k_power_sum(const float* __restrict__ gpart, int chunks, int n,
 }
 
 // End of round t: v = g / ||g||, and in block 0 the stop rule (power_stop) and the
-// estimate.  A block that already sees this round's `done` may skip its part of v,
-// which no later round reads.
+// estimate.  Block 0 may set `done` to t while other blocks start, hence the rule that
+// takes no notice of this launch's own round.
 __global__ void k_power_scale(float* __restrict__ v, int n, const double* __restrict__ part,
                               PowerState* st, int t, int max_iter, double tol, double cap) {
   __shared__ double sh[32];
-  if (st->done) return;
+  if (power_round_over(st->done, t)) return;
   const double nrm = sqrt(sum_to_all(part, gridDim.x, sh));
   const double inv = nrm > 0 ? 1.0 / nrm : 0.0;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)

@@ -46,3 +46,21 @@ int main() {
             assert start % 16 == 0 and start >= end, (m, n, za)
             end = start + length
         assert end <= total, (m, n, za)
+
+
+def test_power_round_decides_alike_before_and_after_its_own_end(run_cpp):
+    """The launch of round t may read `done` before or after its first block writes t: both
+    must run the round.  A later round's launches stop; a running iteration's do not."""
+    lines = run_cpp(r"""
+#include <cstdio>
+#include "rules.h"
+int main() {
+  for (int done = 0; done < 6; ++done)
+    for (int t = 1; t < 6; ++t)
+      std::printf("%d %d %d\n", done, t, (int)mpax::power_round_over(done, t));
+}
+""")
+    over = {(d, t): o for d, t, o in (map(int, line.split()) for line in lines if line)}
+    for t in range(1, 6):
+        assert over[0, t] == over[t, t] == 0
+        assert all(over[d, t] == 1 for d in range(1, t))
