@@ -8,20 +8,46 @@
 namespace mpax {
 
 // ---- rows by lane groups ------------------------------------------------------------
-// A warp takes four consecutive rows: those of at most kGroupRow entries side by side,
-// eight lanes each, the longer ones one after another with all lanes.  With a warp per
-// row most lanes idled on rows of a few entries (a fifth of a million rows of one or two
-// in a power-law matrix), and each row paid a five-step tree of the whole warp.
+// A warp takes four consecutive rows of at most kGroupRow entries side by side, eight lanes
+// each.  With a warp per row most lanes idled on rows of a few entries (a fifth of a million
+// rows of one or two in a power-law matrix), and each row paid a five-step tree of the whole
+// warp.  Longer rows come from a list (LongRows), a warp each: they often stand together (the
+// coupling rows of a model), and one warp that took four of them in turn held up the launch
+// (preparation of an LP of 20 rows of 100,000 entries 67.8 -> 20.4 ms).
 constexpr int kGroup = 8, kGroupRows = 32 / kGroup, kGroupRow = 64;
 
-// f(p, k) on every entry p of this warp's rows; k = (entry's place in its row) % 32 tells
-// which of the row's 32 strided partial sums it belongs to.  done(i, wide) ends row i:
-// called by the eight lanes of a short row's group (wide = false) or by the whole warp.
+// The rows of a matrix with more than kGroupRow entries, in no particular order.
+struct LongRows {
+  const int* n;    // their number, on the device; nullptr: there are none
+  const int* row;
+};
+
+// Rows i of the block's threads with more than kGroupRow entries are appended to n, row.
+__device__ __forceinline__ void append_long(const int* __restrict__ rp, int rows, long long i,
+                                            int* n, int* row) {
+  const bool is_long = i < rows && rp[i + 1] - rp[i] > kGroupRow;
+  const unsigned longs = __ballot_sync(0xffffffffu, is_long);
+  if (longs == 0) return;
+  const int lane = threadIdx.x & 31;
+  int at = lane == 0 ? atomicAdd(n, __popc(longs)) : 0;
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (is_long) row[at + __popc(longs & ((1u << lane) - 1u))] = (int)i;
+}
+__global__ void find_long(const int* __restrict__ rp, int rows, int* n, int* row) {
+  append_long(rp, rows, (long long)blockIdx.x * blockDim.x + threadIdx.x, n, row);
+}
+
+// f(i, p, k) on every entry p of this warp's rows i; k = (entry's place in its row) / 8 % 4
+// tells which of the row's 32 strided partial sums it belongs to.  done(i, valid, wide) ends
+// row i: called by all lanes, for a short row of the lane's group (wide = false) or one row
+// of the whole warp.
 template <class F, class Done>
-__device__ __forceinline__ void for_rows(const int* __restrict__ rp, int rows, F f, Done done) {
+__device__ __forceinline__ void for_rows(const int* __restrict__ rp, int rows, LongRows lr, F f,
+                                         Done done) {
   const int lane = threadIdx.x & 31, gl = lane & (kGroup - 1);
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
+  const int nl = lr.n ? *lr.n : 0;
   for (long long r0 = (long long)warp * kGroupRows; r0 < rows; r0 += (long long)nw * kGroupRows) {
     const bool in = r0 + lane / kGroup < rows;
     const int i = in ? (int)r0 + lane / kGroup : 0;
@@ -32,16 +58,12 @@ __device__ __forceinline__ void for_rows(const int* __restrict__ rp, int rows, F
     }
     __syncwarp();
     done(i, !is_long && in, false);
-    unsigned longs = __ballot_sync(0xffffffffu, is_long && gl == 0);
-    while (longs) {
-      const int src = __ffs(longs) - 1;
-      longs &= longs - 1;
-      const int il = (int)r0 + src / kGroup;
-      const int bl = __shfl_sync(0xffffffffu, b, src), el = __shfl_sync(0xffffffffu, e, src);
-      for (int p = bl + lane; p < el; p += 32) f(il, p, 0);
-      __syncwarp();
-      done(il, true, true);
-    }
+  }
+  for (int t = warp; t < nl; t += nw) {
+    const int i = lr.row[t], e = rp[i + 1];
+    for (int p = rp[i] + lane; p < e; p += 32) f(i, p, 0);
+    __syncwarp();
+    done(i, true, true);
   }
 }
 
@@ -68,11 +90,12 @@ struct RowSum {
 
 // Sum of |K_ij| over the rows; values through `perm` (columns of A as rows of A^T).
 __global__ void row_abssum(const int* __restrict__ rp, const double* __restrict__ val,
-                           const int* __restrict__ perm, int rows, double* __restrict__ out) {
+                           const int* __restrict__ perm, int rows, LongRows lr,
+                           double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   RowSum sum;
   for_rows(
-      rp, rows,
+      rp, rows, lr,
       [&](int, int p, int k) {
         const double v = fabs(val[perm[p]]);
 #pragma unroll
@@ -96,14 +119,15 @@ __global__ void row_abssum(const int* __restrict__ rp, const double* __restrict_
 // 182 us by groups; 2M entries in 100,000 rows of about 20: 59 -> 25 us.
 template <bool SUM>
 __global__ void scale_pass(const int* __restrict__ rp, const int* __restrict__ col,
-                           double* __restrict__ val, int rows, const double* __restrict__ dr,
-                           const double* __restrict__ dc, double* __restrict__ rownorm,
+                           double* __restrict__ val, int rows, LongRows lr,
+                           const double* __restrict__ dr, const double* __restrict__ dc,
+                           double* __restrict__ rownorm,
                            unsigned long long* __restrict__ colmax) {
   const int lane = threadIdx.x & 31;
   RowSum sum;
   unsigned long long mx = 0ull;
   for_rows(
-      rp, rows,
+      rp, rows, lr,
       [&](int i, int p, int k) {
         double v = val[p];
         if (SUM ? dr != nullptr : true) {
@@ -169,12 +193,13 @@ __global__ void factor_update(double* __restrict__ rnorm, int m, double* __restr
 }
 
 // K_ij <- (K_ij * dr_i) * dc_j  (src may differ from dst: start from the original;
-// dr or dc may be nullptr = all ones)
+// dc may be nullptr = all ones)
 __global__ void apply_scale(const int* __restrict__ rp, const int* __restrict__ col,
                             const double* __restrict__ src, double* __restrict__ dst, int rows,
-                            const double* __restrict__ dr, const double* __restrict__ dc) {
+                            LongRows lr, const double* __restrict__ dr,
+                            const double* __restrict__ dc) {
   for_rows(
-      rp, rows,
+      rp, rows, lr,
       [&](int i, int p, int) { dst[p] = dc ? (src[p] * dr[i]) * dc[col[p]] : src[p] * dr[i]; },
       [](int, bool, bool) {});
 }
@@ -200,9 +225,17 @@ __global__ void q_diagonal_add(const int* __restrict__ qrp, const int* __restric
   out[j] += s;
 }
 
-__global__ void fill_ones(double* a, int k) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < k) a[i] = 1.0;
+// D = 1, and the long rows of A and A^T (nl: their two numbers, zero before; nullptr: none).
+__global__ void scaling_start(int m, double* __restrict__ Dr, int n, double* __restrict__ Dc,
+                              const int* __restrict__ rp, const int* __restrict__ rpt, int* nl,
+                              int* lm, int* ln) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < m) Dr[t] = 1.0;
+  if (t < n) Dc[t] = 1.0;
+  if (nl) {
+    append_long(rp, m, t, nl, lm);
+    append_long(rpt, n, t, nl + 1, ln);
+  }
 }
 
 __global__ void inv_vec(const double* __restrict__ a, double* __restrict__ b, int k) {
@@ -219,19 +252,25 @@ __global__ void scale_diag(const double* __restrict__ D, const double* __restric
 
 static int grid_for(long long k) { return (int)std::max(1LL, (k + 255) / 256); }
 // Four rows per warp (up to 2^21 warps, then grid-stride): every row's dependent load
-// chain (row pointer, values and columns, the gathered factor) is in flight at once.
+// chain (row pointer, values and columns, the gathered factor) is in flight at once.  Few
+// rows get a warp each, should they be long.
+constexpr int kFewRows = 152 * 64;  // one warp each fills the GPU
 static int warp_grid(int rows) {
-  const int warps = std::max(1, std::min((rows + kGroupRows - 1) / kGroupRows, 1 << 21));
-  return (warps + 7) / 8;
+  const int warps = std::max((rows + kGroupRows - 1) / kGroupRows, std::min(rows, kFewRows));
+  return (std::max(1, std::min(warps, 1 << 21)) + 7) / 8;
 }
 
 cudaError_t compute_scaling(ProblemData& P, int ruiz_iters, bool pock_chambolle) {
   cudaStream_t s = P.s;
   const int m = P.m, n = P.n;
-  if (m) fill_ones<<<grid_for(m), 256, 0, s>>>(P.Dr, m);
-  if (n) fill_ones<<<grid_for(n), 256, 0, s>>>(P.Dc, n);
-  if (P.nnz) cudaMemcpyAsync(P.val_s, P.val, sizeof(double) * P.nnz, cudaMemcpyDeviceToDevice, s);
   const bool have = (P.nnz > 0 && m > 0 && n > 0);
+  // tmp_rows: the numbers of long rows of A and A^T, then the rows
+  int *nl = P.tmp_rows, *lm = nl + 2, *ln = lm + m;
+  if (have) cudaMemsetAsync(nl, 0, 2 * sizeof(int), s);
+  scaling_start<<<grid_for(std::max(m, n)), 256, 0, s>>>(m, P.Dr, n, P.Dc, P.A.rp, P.At.rp,
+                                                         have ? nl : nullptr, lm, ln);
+  const LongRows la{nl, lm}, lat{nl + 1, ln};
+  if (P.nnz) cudaMemcpyAsync(P.val_s, P.val, sizeof(double) * P.nnz, cudaMemcpyDeviceToDevice, s);
   const int mf = have ? m : 0;  // rows whose factors change
   const double* qd = nullptr;
   if (P.is_qp && n) {
@@ -249,7 +288,7 @@ cudaError_t compute_scaling(ProblemData& P, int ruiz_iters, bool pock_chambolle)
     cudaMemsetAsync(nc, 0, sizeof(double) * n, s);
     if (have)
       scale_pass<false><<<warp_grid(m), 256, 0, s>>>(
-          P.A.rp, P.A.col, P.val_s, m, pending ? fr : nullptr, pending ? fc : nullptr, nr,
+          P.A.rp, P.A.col, P.val_s, m, la, pending ? fr : nullptr, pending ? fc : nullptr, nr,
           reinterpret_cast<unsigned long long*>(nc));
     std::swap(fr, nr);
     std::swap(fc, nc);
@@ -259,10 +298,10 @@ cudaError_t compute_scaling(ProblemData& P, int ruiz_iters, bool pock_chambolle)
   if ((have || qd) && pock_chambolle) {
     if (have) {
       // apply the last Ruiz factors while summing rows; columns through A^T
-      scale_pass<true><<<warp_grid(m), 256, 0, s>>>(P.A.rp, P.A.col, P.val_s, m,
+      scale_pass<true><<<warp_grid(m), 256, 0, s>>>(P.A.rp, P.A.col, P.val_s, m, la,
                                                     pending ? fr : nullptr,
                                                     pending ? fc : nullptr, nr, nullptr);
-      row_abssum<<<warp_grid(n), 256, 0, s>>>(P.At.rp, P.val_s, P.permT, n, nc);
+      row_abssum<<<warp_grid(n), 256, 0, s>>>(P.At.rp, P.val_s, P.permT, n, lat, nc);
     } else {
       cudaMemsetAsync(nc, 0, sizeof(double) * n, s);
     }
@@ -270,17 +309,21 @@ cudaError_t compute_scaling(ProblemData& P, int ruiz_iters, bool pock_chambolle)
   }
   // the scaled matrix from the original values and the accumulated factors
   if (have)
-    apply_scale<<<warp_grid(m), 256, 0, s>>>(P.A.rp, P.A.col, P.val, P.val_s, m, P.Dr, P.Dc);
+    apply_scale<<<warp_grid(m), 256, 0, s>>>(P.A.rp, P.A.col, P.val, P.val_s, m, la, P.Dr, P.Dc);
   if (m) inv_vec<<<grid_for(m), 256, 0, s>>>(P.Dr, P.invDr, m);
   if (n) inv_vec<<<grid_for(n), 256, 0, s>>>(P.Dc, P.invDc, n);
   if (P.is_qp) {
     if (n) scale_diag<<<grid_for(n), 256, 0, s>>>(P.D, P.Dc, n, P.D_s);
-    if (P.f_nnz)
-      apply_scale<<<warp_grid(n), 256, 0, s>>>(P.F.rp, P.F.col, P.fval, P.fval_s, n, P.Dc,
-                                                nullptr);  // F~ = diag(Dc) F
-    if (P.q_general && P.Q.nnz)  // Q~ = diag(Dc) Q diag(Dc)
-      apply_scale<<<warp_grid(n), 256, 0, s>>>(P.Q.rp, P.Q.col, P.qval, P.qval_s, n, P.Dc,
-                                                P.Dc);
+    auto scale = [&](const Csr& K, const double* src, double* dst, const double* dc) {
+      if (K.cols > kGroupRow) {  // its long rows, in place of those of A
+        cudaMemsetAsync(nl, 0, sizeof(int), s);
+        find_long<<<grid_for(n), 256, 0, s>>>(K.rp, n, nl, nl + 1);
+      }
+      apply_scale<<<warp_grid(n), 256, 0, s>>>(
+          K.rp, K.col, src, dst, n, LongRows{K.cols > kGroupRow ? nl : nullptr, nl + 1}, P.Dc, dc);
+    };
+    if (P.f_nnz) scale(P.F, P.fval, P.fval_s, nullptr);                  // F~ = diag(Dc) F
+    if (P.q_general && P.Q.nnz) scale(P.Q, P.qval, P.qval_s, P.Dc);      // diag(Dc) Q diag(Dc)
   }
   return cudaGetLastError();
 }
