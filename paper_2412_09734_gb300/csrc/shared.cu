@@ -52,10 +52,18 @@ dim3 grid2d(long long len, int B) {
   return dim3((unsigned)bx, (unsigned)std::max(1, std::min(B, 65535)));
 }
 
+// Threads of a block that walks the `len` items of one instance: whole warps, no more than
+// there are items.  A block of a small instance holds its SM for one chain of memory round
+// trips however few of its threads work, so the blocks in flight count: 20,000 instances of
+// 8 x 12, 640 iterations, 48.0 ms with 256 threads, 37.5 ms with a warp.
+int row_threads(long long len, int most) {
+  return (int)std::max(32LL, std::min((long long)most, (len + 31) / 32 * 32));
+}
 // Grid of the updates: V coordinates per thread and pass, x over the coordinates of an
 // instance, y over the instances.
-dim3 update_grid(long long len, int B, int V) {
-  const long long bx = std::max(1LL, std::min(1024LL, (len + 256LL * V - 1) / (256LL * V)));
+dim3 update_grid(long long len, int B, int V, int threads) {
+  const long long per = (long long)threads * V;
+  const long long bx = std::max(1LL, std::min(1024LL, (len + per - 1) / per));
   return dim3((unsigned)bx, (unsigned)std::max(1, std::min(B, 65535)));
 }
 // Chunks of the check reductions of B instances of `len` coordinates: blocks of at
@@ -386,7 +394,7 @@ __device__ __forceinline__ void sum_parts(const float* part, int chunks, int len
 // primal: T = A~^T Y; x = w + (anchor - w)/(k+1); x^ = proj(x - tau (c~ - T));
 // w <- 2 x^ - x (BF: also split for the next product).  Check iterations store x^ and x.
 // tpart (B = 1 only): T is the sum of the GEMV's tchunks partials, in order.
-// Grid: x over V coordinates of an instance per thread, y over instances (grid2d).
+// Grid: x over V coordinates of an instance per thread, y over instances (update_grid).
 template <int V, bool BF>
 __global__ void k_primal(Vecs v, const float2* __restrict__ halpern, int check,
                          const float* __restrict__ tpart, int tchunks) {
@@ -462,27 +470,19 @@ __global__ void k_dual(Vecs v, const float2* __restrict__ halpern, int check,
 // the iterates starts on 16 bytes.
 void launch_primal(const Vecs& v, bool bf, const float2* halpern, int check, const float* tpart,
                    int tchunks, cudaStream_t s) {
-  if (v.n % 4 == 0) {
-    const dim3 g = update_grid(v.n, v.B, 4);
-    if (bf) k_primal<4, true><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
-    else k_primal<4, false><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
-  } else {
-    const dim3 g = update_grid(v.n, v.B, 1);
-    if (bf) k_primal<1, true><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
-    else k_primal<1, false><<<g, 256, 0, s>>>(v, halpern, check, tpart, tchunks);
-  }
+  const int V = v.n % 4 == 0 ? 4 : 1, t = row_threads((v.n + V - 1) / V, 256);
+  const dim3 g = update_grid(v.n, v.B, V, t);
+  auto kernel = V == 4 ? (bf ? k_primal<4, true> : k_primal<4, false>)
+                       : (bf ? k_primal<1, true> : k_primal<1, false>);
+  kernel<<<g, t, 0, s>>>(v, halpern, check, tpart, tchunks);
 }
 void launch_dual(const Vecs& v, bool bf, const float2* halpern, int check, const float* spart,
                  int schunks, cudaStream_t s) {
-  if (v.m % 4 == 0) {
-    const dim3 g = update_grid(v.m, v.B, 4);
-    if (bf) k_dual<4, true><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
-    else k_dual<4, false><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
-  } else {
-    const dim3 g = update_grid(v.m, v.B, 1);
-    if (bf) k_dual<1, true><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
-    else k_dual<1, false><<<g, 256, 0, s>>>(v, halpern, check, spart, schunks);
-  }
+  const int V = v.m % 4 == 0 ? 4 : 1, t = row_threads((v.m + V - 1) / V, 256);
+  const dim3 g = update_grid(v.m, v.B, V, t);
+  auto kernel = V == 4 ? (bf ? k_dual<4, true> : k_dual<4, false>)
+                       : (bf ? k_dual<1, true> : k_dual<1, false>);
+  kernel<<<g, t, 0, s>>>(v, halpern, check, spart, schunks);
 }
 
 // Partial sums of a check in FP64: block (c, k) takes chunk c of the coordinates and
@@ -1437,8 +1437,9 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
   sh->prep_seconds =
       std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   // ---- per-instance initial state --------------------------------------------------
-  k_colnorm<<<B, 1024, 0, s>>>(sh->C0, sh->Dc, n, sh->cns);
-  k_colnorm<<<B, 1024, 0, s>>>(sh->C0, nullptr, n, sh->cn);
+  const int ct = row_threads(n, 1024);
+  k_colnorm<<<B, ct, 0, s>>>(sh->C0, sh->Dc, n, sh->cns);
+  k_colnorm<<<B, ct, 0, s>>>(sh->C0, nullptr, n, sh->cn);
   k_bound_norm<<<1, 512, 0, s>>>(sh->lc, sh->uc, sh->Dr, m, sh->scal);
   double bn[2];
   cudaMemcpyAsync(bn, sh->scal, sizeof(bn), cudaMemcpyDeviceToHost, s);

@@ -291,3 +291,52 @@ def test_shared_fp32_product_tiles_match_oracle(C, m, n, B):
             eps_primal_infeasible=0.0, eps_dual_infeasible=0.0, **opts))
         assert rel_inf(X[k], ref.x) <= 1e-5, k
         assert rel_inf(Y[k], ref.y) <= 1e-5, k
+
+
+# The updates run blocks of whole warps, no wider than an instance has items: 1, 31 and 33
+# items per thread group, four coordinates per thread (multiples of four) and one.
+@pytest.mark.parametrize("m,n", [(3, 1), (4, 12), (8, 128), (31, 132), (33, 124), (132, 33)])
+def test_shared_narrow_instances_match_oracle(C, m, n):
+    B = 40
+    d = shared_dense_lp_batch(m, n, B, seed=m * 7 + n, bound_frac=0.5)
+    opts = dict(eps_abs=1e-14, eps_rel=1e-14, iteration_limit=64, power_max_iter=0)
+    h = C.mpax_lp_shared_create(m, n, B, d["A"], d["C"], d["b"], d["b"], d["l"], d["u"])
+    try:
+        C.mpax_shared_solve(h, C.mpax_options_default(fp64_continuation=0, **opts), True)
+        X, Y = C.mpax_shared_get_solution(h, m, n, B)
+    finally:
+        C.mpax_shared_destroy(h)
+    for k in (0, B - 1):
+        ref = O.solve_lp(_oracle_problem(d, k), O.Options(
+            eps_primal_infeasible=0.0, eps_dual_infeasible=0.0, **opts))
+        assert rel_inf(X[k], ref.x) <= 1e-5, k
+        assert rel_inf(Y[k], ref.y) <= 1e-5, k
+
+
+def test_shared_many_tiny_instances_gain_from_four_coordinates_a_thread(C):
+    """20,000 instances of 12 columns (four coordinates per thread) take at most the ratio
+    of the columns longer than those of 11 (one per thread)."""
+    import time
+
+    import torch
+    best = {}
+    for n in (11, 12):
+        rng = np.random.default_rng(n)
+        A = rng.standard_normal((8, n)).astype(np.float32)
+        b = A.astype(np.float64) @ rng.random(n)
+        h = C.mpax_lp_shared_create(8, n, 20000, A, rng.standard_normal((20000, n)), b, b,
+                                    np.zeros(n), np.ones(n))
+        opts = C.mpax_options_default(iteration_limit=640, eps_abs=1e-14, eps_rel=1e-14,
+                                      power_max_iter=0, fp64_continuation=0)
+        try:
+            ts = []
+            for _ in range(5):
+                torch.cuda.synchronize()
+                t = time.perf_counter()
+                C.mpax_shared_solve(h, opts, True)
+                torch.cuda.synchronize()
+                ts.append(time.perf_counter() - t)
+        finally:
+            C.mpax_shared_destroy(h)
+        best[n] = min(ts)
+    assert best[12] <= best[11] * 12 / 11
