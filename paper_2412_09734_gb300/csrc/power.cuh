@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "rules.h"
 #include "sync.cuh"
 
 namespace mpax {
@@ -52,7 +53,7 @@ __device__ __forceinline__ bool grid_sync(const GridBar& b, unsigned& phase) {
     for (unsigned n = 0;; ++n) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(b.w) : "memory");
-      if (v >= phase) break;
+      if (barrier_open(v, phase)) break;
       if ((n & 255u) == 255u) {
         const unsigned long long t = globaltimer_ns();
         if (t0 == 0) t0 = t;

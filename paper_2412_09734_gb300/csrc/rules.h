@@ -16,4 +16,8 @@ namespace mpax {
 // block that disagreed would leave the others alone at the block's barriers.
 MPAX_RULE bool power_round_over(int done, int t) { return done != 0 && done != t; }
 
+// Whether a barrier that waits for `phase` arrivals in all is open at `arrived`.  Both count
+// up modulo 2^32 (a launch of many million rounds passes it), never more than 2^31 apart.
+MPAX_RULE bool barrier_open(unsigned arrived, unsigned phase) { return (int)(arrived - phase) >= 0; }
+
 }  // namespace mpax
