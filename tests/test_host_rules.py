@@ -71,6 +71,7 @@ def test_barrier_opens_with_its_last_arrival_past_the_counter_s_range_too(run_cp
     from then on while the next barrier fills, on both sides of 2^32 arrivals."""
     lines = run_cpp(r"""
 #include <cstdio>
+#include <initializer_list>
 #include "rules.h"
 int main() {
   const unsigned blocks = 152;
