@@ -881,13 +881,16 @@ class Engine final : public EngineBase {
     }
     return cudaSuccess;
   }
-  // A barrier of power_rounds that gave up: cudaErrorTimeout, and the words are zeroed.
+  // A barrier of power_rounds that gave up: cudaErrorTimeout.  Its words are zeroed, and the
+  // arrival counters of the sliced rows: CTAs that went on may have taken part of a row.
   cudaError_t barrier_error() {
     unsigned b = 0;
     cudaError_t e = cudaMemcpyAsync(&b, bar_.w + 2, sizeof(b), cudaMemcpyDeviceToHost, P_->s);
     if (!e) e = cudaStreamSynchronize(P_->s);
     if (e || !b) return e;
     if ((e = cudaMemsetAsync(bar_.w, 0, sizeof(unsigned) * kGridBarWords, P_->s))) return e;
+    for (Sched* q : {&P_->schedA, &P_->schedAt, &P_->schedF, &P_->schedFt, &P_->schedQ})
+      if (q->cnt && (e = cudaMemsetAsync(q->cnt, 0, sizeof(int) * q->n_items, P_->s))) return e;
     return cudaErrorTimeout;
   }
 

@@ -14,8 +14,9 @@
 // and go through L1.  The scalars of a round are formed by one thread: a double division
 // or root on every thread would take the FP64 pipe (16 cycles per warp instruction) longer
 // than the products of a small problem.  The barrier is bounded: a wait that gives up sets
-// the error word, its CTA returns, the others follow within their own limit, and the
-// solve reports MPAX_ERR_DEVICE_TIMEOUT.
+// the error word, its CTA returns, the others follow within their own limit (each decides by
+// its own wait alone, so that its threads decide alike), the host restores the words and
+// counters that the launch left behind, and the solve reports MPAX_ERR_DEVICE_TIMEOUT.
 #pragma once
 
 #include <algorithm>
@@ -39,8 +40,9 @@ struct GridBar {
 constexpr int kGridBarWords = 3;
 
 // All CTAs of the grid (all resident: cooperative launch); phase counts this CTA's
-// arrivals.  False when the wait gave up.
-__device__ __forceinline__ bool grid_sync(const GridBar& b, unsigned& phase) {
+// arrivals.  False when the wait gave up, after `limit_ns` of the device clock.
+__device__ __forceinline__ bool grid_sync(const GridBar& b, unsigned& phase,
+                                          unsigned long long limit_ns = kWaitNs) {
   __shared__ int s_ok;
   __syncthreads();
   if (gridDim.x == 1) return true;
@@ -57,7 +59,7 @@ __device__ __forceinline__ bool grid_sync(const GridBar& b, unsigned& phase) {
       if ((n & 255u) == 255u) {
         const unsigned long long t = globaltimer_ns();
         if (t0 == 0) t0 = t;
-        if (t - t0 > kWaitNs) {
+        if (t - t0 > limit_ns) {
           atomicExch(b.w + 2, 1u);
           ok = 0;
           break;
@@ -135,7 +137,6 @@ __global__ void __launch_bounds__(32 * kRoundWarps, 1)
   __shared__ double sh[32];
   __shared__ double s_scale, s_nu;
   __shared__ int s_stop;
-  if (*(volatile unsigned*)(bar.w + 2)) return;
   unsigned phase = 0;
   double prev = 0.0, d_prev = 0.0;  // thread 0's
   if (threadIdx.x == 0) {
