@@ -103,14 +103,46 @@ struct BatchArgs {
   long long stage_cap;  // bytes of the shared pool an instance may stage whole (0: none)
 };
 
-__device__ __forceinline__ double bsum(double v, double* sh) {
-  v = block_sum(v, sh);
+// A thread's share of a sum over an instance.  The order of the sum is that of a CTA of
+// kBatchThreads threads whatever the launch: with half of them (kFold = 2) a thread keeps the
+// shares of two, so an instance's result does not depend on the batch it is in.
+template <int kFold>
+struct Share {
+  double v[kFold] = {};
+  // x of the item that this thread takes in its pass number `pass`
+  __device__ __forceinline__ void add(int pass, double x) {
+    if constexpr (kFold == 1) {
+      v[0] += x;
+    } else {
+      if (pass & 1) v[1] += x;
+      else v[0] += x;
+    }
+  }
+};
+
+// The sum over the block, to every thread.  Warps without a share skip theirs: a step of the
+// tree takes the FP64 pipe 16 cycles a warp.
+template <int kFold>
+__device__ __forceinline__ double bsum(const Share<kFold>& s, double* sh) {
   __shared__ double bc;
-  if (threadIdx.x == 0) bc = v;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  double part[kFold];
+#pragma unroll
+  for (int f = 0; f < kFold; ++f) {
+    const bool any = __any_sync(0xffffffffu, __double_as_longlong(s.v[f]) != 0);
+    part[f] = any ? warp_sum(s.v[f]) : 0.0;
+  }
   __syncthreads();
-  const double r = bc;
+#pragma unroll
+  for (int f = 0; f < kFold; ++f)
+    if (lane == 0) sh[w + f * warps] = part[f];
   __syncthreads();
-  return r;
+  if (w == 0) {
+    const double v = warp_sum(lane < kFold * warps ? sh[lane] : 0.0);
+    if (lane == 0) bc = v;
+  }
+  __syncthreads();
+  return bc;
 }
 
 template <typename T>
@@ -275,8 +307,8 @@ struct Inst {
 // iterate vector -- is copied into the shared pool first, so the loop touches
 // global memory only at checks (the unscaled data) and at the end.  Otherwise
 // the two gathered vectors sit at ys, xs (shared or global) and the rest is
-// read in place.  kSorted: rows by length (RowsSorted), else CSR.
-template <typename T, bool kStage, bool kSorted>
+// read in place.  kSorted: rows by length (RowsSorted), else CSR.  kFold: see Share.
+template <typename T, bool kStage, bool kSorted, int kFold>
 __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* ys, T* xs,
                                                double* sh, unsigned long long t_launch) {
   static_assert(kSorted || !kStage, "only sorted instances are staged");
@@ -341,13 +373,17 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   auto row_of = [&](int i) { return m0 + (kSorted ? a.permm[m0 + i] : i); };
   auto col_of = [&](int j) { return n0 + (kSorted ? a.permn[n0 + j] : j); };
   auto none = [](int) { return 0; };
+  // the pass in which a thread meets coordinate i in a loop over the block, and row i in each()
+  constexpr int kT = kBatchThreads<T> / kFold;
+  auto pass = [](int i) { return i / kT; };
+  auto row_pass = [](int i) { return i / (kSorted ? kT : kT / kLPR); };
   const bool has_rows = a.rp[m0 + mb] > a.rp[m0];
 
   // ---- power iteration for ||A~_b||_2 from the common start vector ----------
-  double ss0 = 0.0;
+  Share<kFold> ss0;
   for (int j = threadIdx.x; j < nb; j += blockDim.x) {
     const double r = power_start_raw(j);
-    ss0 += r * r;
+    ss0.add(pass(j), r * r);
   }
   const double inv0 = 1.0 / sqrt(fmax(bsum(ss0, sh), 1e-300));
   for (int j = threadIdx.x; j < nb; j += blockDim.x)
@@ -358,10 +394,10 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   for (int t = 1; has_rows && t <= a.power_max_iter; ++t) {
     A.each(xs, none, [&](int i, T s, int) { ys[i] = s; });
     __syncthreads();
-    double acc = 0.0;
+    Share<kFold> acc;
     At.each(ys, none, [&](int j, T s, int) {
       v.gbuf()[j] = s;
-      acc += (double)s * (double)s;
+      acc.add(row_pass(j), (double)s * (double)s);
     });
     const double nrm = sqrt(bsum(acc, sh));
     if (nrm == 0.0) {
@@ -382,17 +418,17 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   }
 
   // ---- initial primal weight, norms of the unscaled data ------------------
-  double s_cs = 0, s_bs = 0, s_c = 0, s_b = 0;
+  Share<kFold> s_cs, s_bs, s_c, s_b;
   for (int j = threadIdx.x; j < nb; j += blockDim.x) {
     const double cs = (double)v.c()[j];
-    s_cs += cs * cs;
-    s_c += a.c0[n0 + j] * a.c0[n0 + j];
+    s_cs.add(pass(j), cs * cs);
+    s_c.add(pass(j), a.c0[n0 + j] * a.c0[n0 + j]);
   }
   for (int i = threadIdx.x; i < mb; i += blockDim.x) {
     const double bs = bound_val((double)v.lc()[i], (double)v.uc()[i]);
     const double bo = bound_val(a.lc0[m0 + i], a.uc0[m0 + i]);
-    s_bs += bs * bs;
-    s_b += bo * bo;
+    s_bs.add(pass(i), bs * bs);
+    s_b.add(pass(i), bo * bo);
   }
   const double ncs = sqrt(bsum(s_cs, sh)), nbs = sqrt(bsum(s_bs, sh));
   const double c_norm = sqrt(bsum(s_c, sh)), b_norm = sqrt(bsum(s_b, sh));
@@ -424,10 +460,14 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   double best_rel = INFINITY;
   while (true) {
     const int len = (int)min((long long)a.check_every, a.iter_limit - total);
-    double P0 = 0, P1 = 0, D0 = 0, D1 = 0;
     const T tt = (T)tau, ss = (T)sigma, iss = (T)(1.0 / sigma);
-    for (int it = 0; it < len; ++it) {
-      const bool chk = (it == len - 1);
+    // Iteration `it` of the block.  The last one, which the check follows, is code of its own:
+    // the sums of the restart rule take registers that the others' loads need.
+    struct Sums {
+      Share<kFold> p0, p1, q0, q1;  // columns, then rows
+    };
+    auto iterate = [&](int it, auto last, Sums& sq) {
+      constexpr bool chk = decltype(last)::value;
       // weights 1/(k+1) and 1/(k+2) of this and the next iterations
       if (it % kCoefs == 0) {
         if (threadIdx.x <= min(kCoefs, len - it)) s_coef[threadIdx.x] = (T)(1.0 / (double)(k + 1 + threadIdx.x));
@@ -447,11 +487,11 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
             const T wn = (T)2 * xh - x;
             v.w()[j] = wn;
             xs[j] = wn;
-            if (chk) {
+            if constexpr (chk) {
               v.xhat()[j] = xh;
               const double d0 = (double)xh - (double)x, d1 = (double)xh - (double)q.x0;
-              P0 += d0 * d0;
-              P1 += d1 * d1;
+              sq.p0.add(row_pass(j), d0 * d0);
+              sq.p1.add(row_pass(j), d1 * d1);
             }
           });
       __syncthreads();
@@ -467,31 +507,38 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
             const T yh = ss * (t - clampv<T>(t, -q.uc, -q.lc));
             const T z = (T)2 * yh - y0;
             ys[i] = z + hb * (q.ya - z);
-            if (chk) {
+            if constexpr (chk) {
               v.yhat()[i] = yh;
               const double d0 = (double)yh - (double)y0, d1 = (double)yh - (double)q.ya;
-              D0 += d0 * d0;
-              D1 += d1 * d1;
+              sq.q0.add(row_pass(i), d0 * d0);
+              sq.q1.add(row_pass(i), d1 * d1);
             }
           });
       __syncthreads();
       ++k;
       ++total;
-    }
+    };
+    Sums sq;
+    for (int it = 0; it + 1 < len; ++it) iterate(it, std::false_type{}, sq);
+    if (len > 0) iterate(len - 1, std::true_type{}, sq);
+    const double P0 = bsum(sq.p0, sh), P1 = bsum(sq.p1, sh);
+    const double D0 = bsum(sq.q0, sh), D1 = bsum(sq.q1, sh);
     // ---- check: relative KKT error of (x^, y^) on the unscaled problem ----
     for (int j = threadIdx.x; j < nb; j += blockDim.x) xs[j] = v.xhat()[j];
     __syncthreads();
-    double K0 = 0, K1 = 0, C0 = 0, C1 = 0, C2 = 0;
+    Share<kFold> r0, r1;
     A.each(xs, none, [&](int i, T s, int) {
       const int g = row_of(i);
       const double ax = (double)s * a.iDr[g];
       const double lo = a.lc0[g], hi = a.uc0[g];
       const double r = ax - fmin(fmax(ax, lo), hi);
-      K0 += r * r;
+      r0.add(row_pass(i), r * r);
       const double y = a.Dr[g] * (double)v.yhat()[i];
-      if (y > 0.0 && isfinite(lo)) K1 += lo * y;
-      if (y < 0.0 && isfinite(hi)) K1 += hi * y;
+      if (y > 0.0 && isfinite(lo)) r1.add(row_pass(i), lo * y);
+      if (y < 0.0 && isfinite(hi)) r1.add(row_pass(i), hi * y);
     });
+    const double K0 = bsum(r0, sh), K1 = bsum(r1, sh);
+    Share<kFold> c0, c1, c2;
     At.each(v.yhat(), none, [&](int j, T s, int) {
       const int g = col_of(j);
       const double aty = (double)s * a.iDc[g];
@@ -501,19 +548,11 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
       const bool lf = isfinite(lo), uf = isfinite(hi);
       const double lh = (lf && uf) ? lam : lf ? fmax(lam, 0.0) : uf ? fmin(lam, 0.0) : 0.0;
       const double rd = lam - lh;
-      C0 += rd * rd;
-      C1 += a.c0[g] * x;
-      C2 += (lf ? lo * fmax(lh, 0.0) : 0.0) + (uf ? hi * fmin(lh, 0.0) : 0.0);
+      c0.add(row_pass(j), rd * rd);
+      c1.add(row_pass(j), a.c0[g] * x);
+      c2.add(row_pass(j), (lf ? lo * fmax(lh, 0.0) : 0.0) + (uf ? hi * fmin(lh, 0.0) : 0.0));
     });
-    P0 = bsum(P0, sh);
-    P1 = bsum(P1, sh);
-    D0 = bsum(D0, sh);
-    D1 = bsum(D1, sh);
-    K0 = bsum(K0, sh);
-    K1 = bsum(K1, sh);
-    C0 = bsum(C0, sh);
-    C1 = bsum(C1, sh);
-    C2 = bsum(C2, sh);
+    const double C0 = bsum(c0, sh), C1 = bsum(c1, sh), C2 = bsum(c2, sh);
     const double nrp = sqrt(K0), nrd = sqrt(C0);
     pobj = C1;
     const double dobj = K1 + C2;
@@ -601,6 +640,7 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
 template <typename T, bool kStaging, int kThreads>
 __global__ void __launch_bounds__(kThreads, kBatchThreads<T> / kThreads)
     batch_lp_kernel(BatchArgs<T> a) {
+  constexpr int kFold = kBatchThreads<T> / kThreads;
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ double sh[32];
   __shared__ int s_inst;
@@ -618,13 +658,13 @@ __global__ void __launch_bounds__(kThreads, kBatchThreads<T> / kThreads)
     // call sites: the whole instance in shared memory; its two gathered vectors in
     // shared memory (shared loads for the gathers), sorted rows or CSR; everything global
     if (kStaging && za > 0 && stage_bytes(mb, nb, za, zt, (int)sizeof(T)) <= a.stage_cap)
-      solve_instance<T, kStaging, true>(a, b, pool, pool + mb, sh, t_launch);
+      solve_instance<T, kStaging, true, kFold>(a, b, pool, pool + mb, sh, t_launch);
     else if (za > 0)
-      solve_instance<T, false, true>(a, b, pool, pool + mb, sh, t_launch);
+      solve_instance<T, false, true, kFold>(a, b, pool, pool + mb, sh, t_launch);
     else if (mb + nb <= a.smem_vec)
-      solve_instance<T, false, false>(a, b, pool, pool + mb, sh, t_launch);
+      solve_instance<T, false, false, kFold>(a, b, pool, pool + mb, sh, t_launch);
     else
-      solve_instance<T, false, false>(a, b, a.gys + a.m_off[b], a.gxs + a.n_off[b], sh, t_launch);
+      solve_instance<T, false, false, kFold>(a, b, a.gys + a.m_off[b], a.gxs + a.n_off[b], sh, t_launch);
   }
 }
 
@@ -1121,7 +1161,7 @@ mpax_status run_batch(mpax_batch* bt, const mpax_options* o, long long* launches
   auto kernel = L.a.stage_cap > 0 ? batch_lp_kernel<T, true, kT> : batch_lp_kernel<T, false, kT>;
   int threads = kT;
   if constexpr (kT > kBatchSmallThreads) {
-    // by the batch's sizes alone, so that staging or not stays the same bits
+    // by the batch's sizes; the results do not depend on it (Share)
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -445,3 +445,34 @@ def test_batch_of_one_tiny_instance(C, lengths, n, stage, prec, eps):
             assert O.kkt(O.problem_from_arrays(inst), x, y, 1.5 * eps, 1.5 * eps)["converged"]
     finally:
         C.mpax_batch_destroy(h)
+
+
+def test_fp32_instance_gives_the_same_bits_in_any_batch(C):
+    """Batches of many small instances run CTAs of half the threads; an instance's iterates,
+    restarts and KKT error are those that it has in a small batch, to the bit: instances of
+    one warp's rows up to several passes of a CTA, and one with a dense row (CSR)."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(21)
+    shapes = [([3] * 20, 30), (list(rng.integers(1, 12, 300)), 400), (list(rng.integers(2, 9, 515)), 1030),
+              (list(rng.integers(2, 7, 1100)), 2300), ([2900] + [2] * 600, 3000)]
+    insts = [_shaped_instance(L, n, 40 + i) for i, (L, n) in enumerate(shapes)]
+    fill = _shaped_instance([4, 5, 6, 7], 12, 60)
+    # two passes of power sums, restarts at checks of their own and a limit that ends between
+    opts = C.mpax_options_default(precision=1, fp64_continuation=0, eps_abs=1e-14, eps_rel=1e-14,
+                                  iteration_limit=1000)
+    got = []
+    for B in (len(insts), 2 * sms, 2 * sms + 1, 2 * sms + 40):
+        d = _pack(insts + [fill] * (B - len(insts)))
+        h = _create(C, d)
+        try:
+            C.mpax_batch_solve(h, opts)
+            _, per = C.mpax_batch_get_stats(h, B)
+            x, y = C.mpax_batch_get_solution(h, int(d["m_off"][-1]), int(d["n_off"][-1]))
+        finally:
+            C.mpax_batch_destroy(h)
+        k = len(insts)
+        got.append((x[:d["n_off"][k]], y[:d["m_off"][k]], per["rel_kkt"][:k]))
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            np.testing.assert_array_equal(a, b)
