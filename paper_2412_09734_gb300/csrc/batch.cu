@@ -1169,8 +1169,7 @@ mpax_status run_batch(mpax_batch* bt, const mpax_options* o, long long* launches
     for (int b = 0; b < bt->B && small; ++b)
       small = bt->h_moff[b + 1] - bt->h_moff[b] + bt->h_noff[b + 1] - bt->h_noff[b] <= kSmallVec;
     if (small) {
-      kernel = L.a.stage_cap > 0 ? batch_lp_kernel<T, true, kBatchSmallThreads>
-                                 : batch_lp_kernel<T, false, kBatchSmallThreads>;
+      kernel = batch_lp_kernel<T, false, kBatchSmallThreads>;  // more instances than are staged
       threads = kBatchSmallThreads;
     }
   }
