@@ -309,10 +309,24 @@ constexpr int kChunks = 128;
 // (0-1 restart metric, 2-5 KKT columns, 6-9 ray columns) then 6 of the A
 // schedule (0-1 restart metric, 2-3 KKT rows, 4-5 ray rows).
 constexpr int kCheckQt = 10, kCheckQa = 6, kCheckQ = kCheckQt + kCheckQa;
+// The norm of the power iteration has one slot, where a single warp would be a long chain of
+// additions: from kLongChunk values per block on, all warps share it (8M values 107 -> 52 us,
+// 1M 16.5 -> 10.4, 200,000 the same).
+constexpr int kLongChunk = 2048;
 __global__ void k_part_reduce(const double* __restrict__ partAt, int nAt, int qt,
                               const double* __restrict__ partA, int nA, int qa,
                               const int* skip, double* __restrict__ out) {
+  __shared__ double sh[32];
   if (skip && *skip) return;
+  if (qt == 1 && qa == 0 && nAt > kChunks * kLongChunk) {
+    const int chunk = (nAt + kChunks - 1) / kChunks;
+    const int lo = blockIdx.x * chunk, hi = min(nAt, lo + chunk);
+    double v = 0;
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) v += partAt[i];
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) out[blockIdx.x] = v;
+    return;
+  }
   for (int q = threadIdx.x >> 5; q < qt + qa; q += blockDim.x >> 5) {
     const double* p = q < qt ? partAt + (size_t)q * nAt : partA + (size_t)(q - qt) * nA;
     const int n = q < qt ? nAt : nA;

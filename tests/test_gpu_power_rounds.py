@@ -51,3 +51,21 @@ def test_single_launch_norms_match_oracle(C, case):
     np.testing.assert_allclose(norms[0][0], nA, rtol=1e-9)
     if p.is_qp:
         np.testing.assert_allclose(norms[0][1], nQ, rtol=1e-9)
+
+
+@pytest.mark.parametrize("rows", [16_800_000, 16_700_000])
+def test_norm_sum_over_very_many_items(C, rows):
+    """0.7 times the identity: every work item (64 rows) adds alike to the norm of the first
+    round, on both sides of the 262,144 items from which all warps of a block share the sum."""
+    import torch
+    n = rows
+    rp = torch.arange(n + 1, dtype=torch.int64, device="cuda")
+    col = torch.arange(n, dtype=torch.int32, device="cuda")
+    one = torch.ones(n, dtype=torch.float64, device="cuda")
+    h = C.mpax_lp_create(n, n, rp, col, 0.7 * one, one, one, one, 0 * one, one)
+    try:
+        C.mpax_prepare(h, C.mpax_options_default(ruiz_iters=0, pock_chambolle=0, spmv_kernel=0))
+        _, _, info = C.mpax_get_scaling(h, n, n)
+    finally:
+        C.mpax_destroy(h)
+    np.testing.assert_allclose(info["norm_A"], 0.7, rtol=1e-12)
