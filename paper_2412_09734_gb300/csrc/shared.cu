@@ -351,7 +351,10 @@ struct Vecs {
 // that takes 16 cycles for a warp, so none may run per coordinate.  Measured on 512
 // instances of 8192 x 16384: with the divisions in the updates 124 us (primal) and
 // 109 us (dual), from this table with 128-bit accesses 32 us (6.3 TB/s) and 13.7 us.
-constexpr int kCoefIters = 256;  // iterations per table
+constexpr int kCoefIters = 256;  // iterations per table, at most
+// Iterations per table of B instances: many instances get a shorter table (a launch of it
+// costs little beside their updates), or it would take 2 KB of memory for each.
+int coef_iters(int B) { return std::max(1, std::min(kCoefIters, (1 << 22) / B)); }
 __global__ void k_coefs(const Inst* __restrict__ inst, int B, int it0, int len,
                         float4* __restrict__ step, float2* __restrict__ halpern) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -876,7 +879,7 @@ struct mpax_shared {
   PowerState* pstate = nullptr;           // power iteration: state and block partials
   double* ppart = nullptr;
   float4* step = nullptr;                 // per-instance step sizes (k_coefs)
-  float2* halpern = nullptr;              // Halpern weights of kCoefIters iterations (k_coefs)
+  float2* halpern = nullptr;              // Halpern weights of coef_iters iterations (k_coefs)
   int chunks = 1;                         // chunks of the check reductions
   Inst* inst = nullptr;
   double *Xout = nullptr, *Yout = nullptr;
@@ -1289,7 +1292,7 @@ mpax_status mpax_lp_shared_create(int32_t m, int32_t n, int32_t B, const float* 
   al(&sh->pstate, 1);
   al(&sh->ppart, kPowerBlocks);
   al(&sh->step, B);
-  al(&sh->halpern, (size_t)kCoefIters * B);
+  al(&sh->halpern, (size_t)coef_iters(B) * B);
   al(&sh->cn, B);
   al(&sh->cns, B);
   al(&sh->inst, B);
@@ -1465,6 +1468,7 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
               sh->yprev, sh->ya, sh->Dr, sh->Dc, sh->iDr, sh->iDc, sh->C0, sh->lc, sh->uc,
               sh->l, sh->u, sh->part};
   long long done_iters = 0;
+  const int table = coef_iters(B);
   // time limit, checked at each KKT check against the host clock
   const long long tl_ns = o->time_limit >= 9.0e9 ? LLONG_MAX : (long long)(o->time_limit * 1e9);
   std::vector<Inst> hi(B);
@@ -1473,9 +1477,9 @@ mpax_status mpax_shared_solve(mpax_shared* sh, const mpax_options* o, int32_t fp
     const int len = (int)std::min<long long>(o->check_every, o->iteration_limit - done_iters);
     for (int it = 0; it < len; ++it) {
       const int chk = (it == len - 1);
-      const float2* hk = sh->halpern + (size_t)(it % kCoefIters) * B;
-      if (it % kCoefIters == 0) {
-        const int cl = std::min(kCoefIters, len - it);
+      const float2* hk = sh->halpern + (size_t)(it % table) * B;
+      if (it % table == 0) {
+        const int cl = std::min(table, len - it);
         k_coefs<<<(B * cl + 255) / 256, 256, 0, s>>>(sh->inst, B, it, cl, sh->step, sh->halpern);
         L += 1;
       }

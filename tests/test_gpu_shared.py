@@ -340,3 +340,28 @@ def test_shared_many_tiny_instances_gain_from_four_coordinates_a_thread(C):
             C.mpax_shared_destroy(h)
         best[n] = min(ts)
     assert best[12] <= best[11] * 12 / 11
+
+
+def test_shared_very_many_instances_use_little_memory_and_the_same_weights(C):
+    """262,144 instances of 3 x 5 take less than 1 KB each on the device, and their step
+    weights, formed for 16 iterations at a time, give the bits of a small batch's, formed at
+    once for the whole block."""
+    import torch
+    m, n, B, few = 3, 5, 1 << 18, 40
+    d = shared_dense_lp_batch(m, n, B, seed=3, bound_frac=0.5)
+    opts = C.mpax_options_default(iteration_limit=400, check_every=200, eps_abs=1e-14, eps_rel=1e-14,
+                                  power_max_iter=0, fp64_continuation=0)
+    X, Y = {}, {}
+    for b in (few, B):
+        before = torch.cuda.mem_get_info()[0]
+        h = C.mpax_lp_shared_create(m, n, b, d["A"], np.ascontiguousarray(d["C"][:b]), d["b"], d["b"],
+                                    d["l"], d["u"])
+        try:
+            if b == B:
+                assert before - torch.cuda.mem_get_info()[0] < 1024 * B
+            C.mpax_shared_solve(h, opts, True)
+            X[b], Y[b] = C.mpax_shared_get_solution(h, m, n, b)
+        finally:
+            C.mpax_shared_destroy(h)
+    np.testing.assert_array_equal(X[few], X[B][:few])
+    np.testing.assert_array_equal(Y[few], Y[B][:few])
