@@ -36,6 +36,7 @@
 #include "../../include/mpax.h"
 #include "umma_host.h"
 #include "common.cuh"
+#include "float_pair.h"
 #include "rules.h"
 #include "sgemm.cuh"
 
@@ -134,12 +135,9 @@ __device__ __forceinline__ void split_vec(const float* v, __nv_bfloat16* hi, __n
 //
 // The pass is bound by HBM (one read, and one write from the second round on) only if
 // it keeps off the FP64 pipe (two lanes per SM and cycle), so the scaled value
-// fl32((a r) c), r and c in FP64, is formed from float pairs: r = rh + rl, c = ch + cl
-// to 48 bits and error-free FP32 products give a r c to within 2^-44.  Where that
-// margin leaves the rounding to a float open (about one value in 10^6), or a product
-// leaves the range in which the pairs are exact, the value is formed in FP64: the
-// result is that of the FP64 products, bit for bit (the BF16 splits of the products
-// that follow turn any other last bit into a 2^-17 one).
+// fl32((a r) c), r and c in FP64, is formed from float pairs (float_pair.h): the result is
+// that of the FP64 products, bit for bit (the BF16 splits of the products that follow turn
+// any other last bit into a 2^-17 one).
 // Measured on 8192 x 16384 (0.54 GB): row maxima 0.79 ms, column maxima 1.88 ms and
 // scaling 1.00 ms before; one pass 0.16 ms (6.5 TB/s) now.
 constexpr int kDenseRows = 64;  // rows of a tile
@@ -154,21 +152,6 @@ struct DensePass {
   __nv_bfloat16 *hi, *lo;       // BF16 split of the result (rows of ldh)
   long long ldh;
 };
-
-__device__ __forceinline__ float scale_pair(float a, float2 r, float2 c, const double* dr,
-                                            const double* dc) {
-  const float p = a * r.x;
-  const float pl = fmaf(a, r.y, fmaf(a, r.x, -p));
-  const float q = p * c.x;
-  const float ql = fmaf(p, c.y, fmaf(pl, c.x, fmaf(p, c.x, -q)));
-  const float ap = fabsf(p), aq = fabsf(q);
-  const float d = aq * 1.1368684e-13f;  // 2^-43
-  const float up = q + (ql + d), dn = q + (ql - d);
-  // (false for NaN, infinities, zeros and values near the ends of the range)
-  if (up == dn && ap > 1e-22f && ap < 1e30f && aq > 1e-22f && aq < 1e30f) return up;
-  if (a == 0.0f) return a;
-  return (float)(((double)a * *dr) * *dc);
-}
 
 template <int V, bool kFactor, bool kMax, bool kWrite, bool kSplit>
 __global__ void __launch_bounds__(256) k_dense_pass(DensePass a) {
@@ -272,11 +255,6 @@ __global__ void __launch_bounds__(kColThreads) k_col_sum(const float* __restrict
   out[j] = acc;
 }
 
-__device__ __forceinline__ float2 float_pair(double d) {
-  const float h = (float)d;
-  return make_float2(h, isfinite(h) ? (float)(d - (double)h) : 0.0f);
-}
-
 // The factors of a finished round, d = 1/sqrt(norm) (1 for an empty row or column),
 // rows then columns: D *= d; d (over dr, dc) and its float pair are stored.  Norms are
 // the float bits nmax (reset to zero for the next round) or, without them, dr and dc.
@@ -293,7 +271,7 @@ __global__ void k_dense_factor(int m, int n, unsigned* __restrict__ nmax, double
   const double d = v > 0.0 ? 1.0 / sqrt(v) : 1.0;
   (row ? Dr : Dc)[i] *= d;
   (row ? dr : dc)[i] = d;
-  (row ? fr : fc)[i] = float_pair(d);
+  (row ? fr : fc)[i] = float_pair<float2>(d);
 }
 
 // The accumulated factors (rows then columns): float pairs and inverses.
@@ -306,7 +284,7 @@ __global__ void k_dense_final(int m, int n, const double* __restrict__ Dr,
   const bool row = t < m;
   const int i = row ? t : t - m;
   const double d = (row ? Dr : Dc)[i];
-  (row ? fr : fc)[i] = float_pair(d);
+  (row ? fr : fc)[i] = float_pair<float2>(d);
   (row ? iDr : iDc)[i] = 1.0 / d;
 }
 

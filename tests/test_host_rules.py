@@ -15,7 +15,7 @@ def run_cpp(tmp_path):
     def go(source):
         src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
         src.write_text(source)
-        subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+        subprocess.run(["g++", "-std=c++17", "-O1", "-ffp-contract=off", "-I", CSRC, str(src), "-o", str(exe)], check=True)
         return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split("\n")
     return go
 
@@ -86,3 +86,40 @@ int main() {
     assert len(lines) > 4000
     for d, is_open in (map(int, line.split()) for line in lines if line):
         assert is_open == (d >= 0), d
+
+
+def test_scaled_value_from_float_pairs_is_the_fp64_product(run_cpp):
+    """Bit for bit, for values and factors over the whole float range and near 1, and for
+    zeros, infinities and NaN."""
+    lines = run_cpp(r"""
+#include <cstdio>
+#include <cstring>
+#include <random>
+#include "float_pair.h"
+struct Pair { float x, y; };
+static long bad = 0;
+static void check(float a, double r, double c) {
+  const float got = mpax::scale_pair(a, mpax::float_pair<Pair>(r), mpax::float_pair<Pair>(c), &r, &c);
+  const float want = (float)(((double)a * r) * c);
+  if (got != got && want != want) return;
+  if (std::memcmp(&got, &want, 4) != 0 && bad++ < 5) std::printf("%a %a %a\n", a, r, c);
+}
+int main() {
+  std::mt19937_64 g(1);
+  std::uniform_real_distribution<double> u(0.0, 1.0);
+  auto pick = [&](double lo, double hi) {
+    return std::ldexp(1.0 + u(g), (int)std::floor(lo + (hi - lo) * u(g)));
+  };
+  for (long i = 0; i < 3000000; ++i) {
+    check((float)pick(-149, 128) * (i & 1 ? 1.0f : -1.0f), pick(-149, 100), pick(-149, 100));
+    check((float)pick(-4, 4), pick(-4, 4), pick(-4, 4));
+    check((float)pick(90, 128), pick(-128, -90), pick(-3, 3));
+  }
+  for (float a : {0.0f, -0.0f, INFINITY, -INFINITY, NAN, 1.0f})
+    for (double r : {0.0, 1.0, 1e-40, 1e30})
+      for (double c : {0.0, 1.0, 1e-40, 1e30})
+        check(a, r, c);
+  std::printf("bad %ld\n", bad);
+}
+""")
+    assert lines[-2] == "bad 0", lines
