@@ -373,6 +373,12 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
   auto row_of = [&](int i) { return m0 + (kSorted ? a.permm[m0 + i] : i); };
   auto col_of = [&](int j) { return n0 + (kSorted ? a.permn[n0 + j] : j); };
   auto none = [](int) { return 0; };
+  // a product of the scaled matrix in the unscaled space: one rounding in FP64; a product of
+  // FP32 sums takes the stored reciprocal, whose rounding lies 2^29 below theirs
+  auto unscale = [](double s, double d, double inv) {
+    if constexpr (sizeof(T) == 8) return s / d;
+    else return s * inv;
+  };
   // the pass in which a thread meets coordinate i in a loop over the block, and row i in each()
   constexpr int kT = kBatchThreads<T> / kFold;
   auto pass = [](int i) { return i / kT; };
@@ -529,7 +535,7 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
     Share<kFold> r0, r1;
     A.each(xs, none, [&](int i, T s, int) {
       const int g = row_of(i);
-      const double ax = (double)s * a.iDr[g];
+      const double ax = unscale((double)s, a.Dr[g], a.iDr[g]);
       const double lo = a.lc0[g], hi = a.uc0[g];
       const double r = ax - fmin(fmax(ax, lo), hi);
       r0.add(row_pass(i), r * r);
@@ -541,7 +547,7 @@ __device__ __forceinline__ void solve_instance(const BatchArgs<T>& a, int b, T* 
     Share<kFold> c0, c1, c2;
     At.each(v.yhat(), none, [&](int j, T s, int) {
       const int g = col_of(j);
-      const double aty = (double)s * a.iDc[g];
+      const double aty = unscale((double)s, a.Dc[g], a.iDc[g]);
       const double x = a.Dc[g] * (double)xs[j];
       const double lam = a.c0[g] - aty;
       const double lo = a.l0[g], hi = a.u0[g];
