@@ -476,3 +476,27 @@ def test_fp32_instance_gives_the_same_bits_in_any_batch(C):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("extra", [0, 1])
+def test_batch_small_instances_iterates_match_oracle(C, extra):
+    """On both sides of two instances per SM, where CTAs of half the threads begin: 64
+    iterations of every kept instance, without a continuation in FP64 that could mend them.
+    1e-5 as in test_batch_iterates_match_oracle."""
+    import torch
+    B = 2 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    d = ragged_lp_batch(B, seed=37, m_lo=20, m_hi=60, density=0.1)
+    opts = dict(iteration_limit=64, eps_abs=1e-14, eps_rel=1e-14, power_max_iter=0)
+    h = _create(C, d)
+    try:
+        C.mpax_batch_solve(h, C.mpax_options_default(precision=1, fp64_continuation=0, **opts))
+        _, per = C.mpax_batch_get_stats(h, B)
+        x, y = C.mpax_batch_get_solution(h, int(d["m_off"][-1]), int(d["n_off"][-1]))
+    finally:
+        C.mpax_batch_destroy(h)
+    assert np.all(per["iterations"] == 64)
+    for b in range(0, B, 19):
+        ref = O.solve_lp(O.problem_from_arrays(d["instances"][b]), O.Options(
+            eps_primal_infeasible=0.0, eps_dual_infeasible=0.0, **opts))
+        assert rel_inf(x[d["n_off"][b]:d["n_off"][b + 1]], ref.x) <= 1e-5, b
+        assert rel_inf(y[d["m_off"][b]:d["m_off"][b + 1]], ref.y) <= 1e-5, b

@@ -69,3 +69,24 @@ def test_norm_sum_over_very_many_items(C, rows):
     finally:
         C.mpax_destroy(h)
     np.testing.assert_allclose(info["norm_A"], 0.7, rtol=1e-12)
+
+
+@pytest.mark.parametrize("case", list(CASES))
+def test_single_launch_runs_and_agrees_with_launched_rounds(C, case):
+    """A caller that names the kernel of the products gets the rounds as launches of their
+    own: the same norms to the 1e-9 of the oracle's, and more launches in all (four a round
+    and at least two rounds against one)."""
+    from paper_2412_09734_gb300.problem import Problem
+    d = CASES[case]()
+    p = Problem.from_dict(d)
+    got = {}
+    for kind in (-1, -1, 0):  # the first solve also times the kernels
+        C.mpax_solve(p.h, C.mpax_options_default(spmv_kernel=kind, iteration_limit=64, eps_abs=1e-14,
+                                                 eps_rel=1e-14))
+        info = C.mpax_get_scaling(p.h, d["m"], d["n"])[2]
+        got[kind] = (info["norm_A"], info["norm_Q"], C.mpax_get_stats(p.h)["kernel_launches"])
+    p.close()
+    np.testing.assert_allclose(got[-1][0], got[0][0], rtol=1e-9)
+    if p.is_qp:
+        np.testing.assert_allclose(got[-1][1], got[0][1], rtol=1e-9)
+    assert got[0][2] >= got[-1][2] + 7 * (2 if p.is_qp else 1)

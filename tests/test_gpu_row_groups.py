@@ -89,3 +89,35 @@ def test_packed_items_cover_every_row_once(C, pattern):
     v = y - A @ (2 * xh - x)  # y^ = v - proj_[0, inf)(v)
     np.testing.assert_allclose(yh, np.minimum(v, 0.0), rtol=1e-12,
                                atol=1e-12 * np.abs(val).sum())
+
+
+# The same patterns with equality rows: y^ = v - proj(v) = v shows the product of every row,
+# and of every column through x^, against a bound of its own.  A row sum of at most 100 terms
+# in FP64 is good to 1.2e-14 of the sum of their magnitudes, and x^ enters the rows' products
+# with that error once more; 1e-13 of the magnitudes is far below a lost or doubled entry.
+@pytest.mark.parametrize("pattern", ["empty", "three", "four", "mixed8", "forty", "bursts"])
+def test_every_row_and_column_product(C, pattern):
+    rng = np.random.default_rng(len(pattern))
+    m, n = 1300, 900
+    lengths = {"empty": np.where(np.arange(m) % 400 < 330, 0, 5),
+               "three": np.full(m, 3), "four": rng.integers(3, 6, m),
+               "mixed8": rng.integers(4, 13, m), "forty": np.full(m, 40),
+               "bursts": np.where((np.arange(m) // 70) % 2 == 0, 0, 60)}[pattern]
+    rp, col, val = _matrix(list(lengths), n, 78)
+    A = sp.csr_matrix((val, col, rp), shape=(m, n))
+    assert max(np.diff(rp).max(), np.bincount(col).max()) <= 100
+    h = C.mpax_lp_create(m, n, rp, col, val, np.ones(n), np.zeros(m), np.zeros(m),
+                         np.full(n, -1e30), np.full(n, 1e30))
+    try:
+        C.mpax_prepare(h, C.mpax_options_default(ruiz_iters=0, pock_chambolle=0, power_max_iter=2))
+        x, y = rng.standard_normal(n), rng.standard_normal(m)
+        C.mpax_set_iterate(h, x, y, x, y, 0, 1.0, 1.0)
+        C.mpax_iterate(h, 1)
+        _, _, xh, yh = C.mpax_get_iterate(h, m, n)
+    finally:
+        C.mpax_destroy(h)
+    ref = x - (1.0 - A.T @ y)
+    bx = 1e-13 * (np.abs(x) + 1.0 + abs(A).T @ np.abs(y))
+    assert np.all(np.abs(xh - ref) <= bx)
+    by = 1e-13 * np.abs(y) + abs(A) @ (1e-13 * np.abs(x) + 3.0 * bx)
+    assert np.all(np.abs(yh - (y - A @ (2.0 * ref - x))) <= by)
