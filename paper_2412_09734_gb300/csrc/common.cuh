@@ -194,6 +194,7 @@ struct HostStatus {
   volatile int termination;
   volatile double rel_kkt;
   volatile double pobj, dobj, primal_res, dual_res, gap, omega;
+  volatile int power_done, power_launch;  // a power iteration's end and progress (power.cuh)
 };
 
 // ---------------------------------------------------------------------------

@@ -673,15 +673,13 @@ class Engine final : public EngineBase {
       }
     }
     st_ = dalloc<DevState>(1, e);
-    bar_.w = dalloc<unsigned>(kGridBarWords, e);
-    csum_ = dalloc<double>(kRoundMaxCtas, e);
+    rs_ = dalloc<RoundState>(2, e);
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev);
     if (*e == cudaSuccess) *e = cudaHostAlloc(&hs_, sizeof(HostStatus), cudaHostAllocMapped);
     if (*e == cudaSuccess) *e = cudaHostGetDevicePointer((void**)&hs_dev_, hs_, 0);
     if (*e == cudaSuccess) *e = cudaMemsetAsync(st_, 0, sizeof(DevState), P->s);
-    if (*e == cudaSuccess) *e = cudaMemsetAsync(bar_.w, 0, sizeof(unsigned) * kGridBarWords, P->s);
   }
 
   ~Engine() override {
@@ -690,7 +688,7 @@ class Engine final : public EngineBase {
     void* bufs[] = {valA_, valAt_, c_,    l_,    u_,    lc_,   uc_,    xbar_, wbuf_,
                     xa_,   xhat_,  xprev_, pv_,  pg_,   y_,    ya_,    yhat_, yprev_,
                     pw_,   x_,     xavg_, xref_, xanc_, yavg_, yanc_,  Ds_,   fval_,
-                    ftval_, uvec_, uvec2_, rayx_, rayy_, qv_, qvec_, qvec2_, st_, bar_.w, csum_};
+                    ftval_, uvec_, uvec2_, rayx_, rayy_, qv_, qvec_, qvec2_, st_, rs_};
     for (void* b : bufs)
       if (b) cudaFree(b);
     if (hs_) cudaFreeHost(hs_);
@@ -750,8 +748,8 @@ class Engine final : public EngineBase {
     T* v = pv_;
     T* g = pg_;
     const int* skip = &st_->pw_done;
-    // all rounds in one launch where the products are small (power.cuh); a caller that
-    // names a kernel of the products gets it
+    // small and medium products have rounds of their own (power.cuh); a caller that names a
+    // kernel of the products gets it
     if (o.spmv_kernel < 0) {
       const bool two = mode == 0 || !P.q_general;
       SpmvArgs<T> a1{}, a2{};
@@ -764,18 +762,11 @@ class Engine final : public EngineBase {
         a1 = fused_args<T>(P.schedFt, P.Ft, ftval_, 0);
         a2 = fused_args<T>(P.schedF, P.F, fval_, 0);
       }
-      const int most = std::max(a1.n_items, a2.n_items);
-      if (a2.n_items > 0 && round_fits(most, sms_)) {
-        const double cap = mode == 0 && o.pock_chambolle ? 1.0 : INFINITY;
-        const cudaError_t e = launch_cooperative(
-            power_rounds<T>, round_ctas(most, sms_), 32 * kRoundWarps, kRoundSmem<T>, s, a1, a2,
-            (int)two, v, g, mode == 0 ? pw_ : uvec_, mode == 1 && two ? (const T*)Ds_ : nullptr,
-            (int)(mode == 0), o.power_tol, cap, (int)o.power_max_iter, csum_, st_, bar_);
-        if (!e) {
-          *launches += 1;
-          return barrier_error();
-        }
-        cudaGetLastError();  // not all CTAs fit at once (a partitioned GPU): launched rounds
+      if (a2.n_items > 0 && round_fits(std::max(a1.n_items, a2.n_items), sms_)) {
+        const RoundRule rule{(int)(mode == 0), o.power_tol,
+                             mode == 0 && o.pock_chambolle ? 1.0 : INFINITY, (int)o.power_max_iter};
+        return rounds(a1, a2, two, v, g, mode == 0 ? pw_ : uvec_,
+                      mode == 1 && two ? (const T*)Ds_ : nullptr, rule, launches);
       }
     }
     for (int t = 1; t <= o.power_max_iter; ++t) {
@@ -821,6 +812,62 @@ class Engine final : public EngineBase {
       }
     }
     return cudaGetLastError();
+  }
+
+  // The rounds of power.cuh.  The host launches round t once launch t - kRoundsAhead runs: far
+  // enough ahead to keep the device busy, and few launches too many at the end.
+  cudaError_t rounds(SpmvArgs<T> a1, SpmvArgs<T> a2, bool two, T* v, T* g, T* w, const T* diag,
+                     const RoundRule& rule, long long* launches) {
+    constexpr int kRoundsAhead = 2, kSmem = kRoundSmem<T>, kThreads = 32 * kRoundWarps;
+    cudaStream_t s = P_->s;
+    cudaError_t e;
+    if (std::max(a1.n_items, a2.n_items) <= kOneCtaItems) {
+      if ((e = allow_smem(power_rounds<T>, kSmem))) return e;
+      power_rounds<T><<<1, kThreads, kSmem, s>>>(a1, a2, (int)two, v, g, w, diag, rule, st_);
+      *launches += 1;
+      return cudaGetLastError();
+    }
+    if ((e = allow_smem(power_step<T, true>, kSmem))) return e;
+    if ((e = allow_smem(power_step<T, false>, kSmem))) return e;
+    // a first product's launch has one CTA more, which ends the round before
+    const int c1 = round_ctas(two ? a1.n_items : a2.n_items, sms_ - 1);
+    const int c2 = round_ctas(a2.n_items, sms_);
+    hs_->power_done = hs_->power_launch = 0;
+    int t = 1;
+    for (; t <= rule.max_iter && !hs_->power_done; ++t) {
+      for (unsigned spin = 1; hs_->power_launch < t - kRoundsAhead && !hs_->power_done; ++spin) {
+        if (spin % 4096) continue;
+        // (a launch that failed reports nothing: the stream has an error or is empty)
+        if ((e = cudaStreamQuery(s)) != cudaErrorNotReady) {
+          if (e) return e;
+          break;
+        }
+        cudaGetLastError();  // "not ready" is no error of a launch
+      }
+      if (two) {
+        power_step<T, true><<<c1 + 1, kThreads, kSmem, s>>>(a1, v, w, nullptr, nullptr, 0, t, a2.part,
+                                                        a2.n_items, rule, rs_, st_, hs_dev_);
+        power_step<T, false><<<c2, kThreads, kSmem, s>>>(a2, w, g, diag, v, 1, t, nullptr, 0, rule,
+                                                         rs_, st_, hs_dev_);
+      } else {  // partial sums in two slots: a launch reads the round's before it
+        a2.q0 = t & 1;
+        power_step<T, true><<<c1 + 1, kThreads, kSmem, s>>>(
+            a2, v, g, nullptr, nullptr, 1, t, a2.part + (size_t)((t - 1) & 1) * a2.n_items,
+            a2.n_items, rule, rs_, st_, hs_dev_);
+      }
+      if ((e = cudaGetLastError())) return e;
+      *launches += two ? 2 : 1;
+      std::swap(v, g);
+    }
+    if (t > rule.max_iter) {
+      SpmvArgs<T> none{};
+      power_step<T, true><<<1, kThreads, kSmem, s>>>(
+          none, nullptr, nullptr, nullptr, nullptr, 0, t,
+          a2.part + (two ? 0 : (size_t)((t - 1) & 1) * a2.n_items), a2.n_items, rule, rs_, st_, hs_dev_);
+      *launches += 1;
+    }
+    if ((e = cudaGetLastError())) return e;
+    return cudaStreamSynchronize(s);  // no launch may still report an end when the next rounds begin
   }
 
   // ---- autotuner: which kernel runs the A and A^T schedules -------------------
@@ -895,19 +942,6 @@ class Engine final : public EngineBase {
     }
     return cudaSuccess;
   }
-  // A barrier of power_rounds that gave up: cudaErrorTimeout.  Its words are zeroed, and the
-  // arrival counters of the sliced rows: CTAs that went on may have taken part of a row.
-  cudaError_t barrier_error() {
-    unsigned b = 0;
-    cudaError_t e = cudaMemcpyAsync(&b, bar_.w + 2, sizeof(b), cudaMemcpyDeviceToHost, P_->s);
-    if (!e) e = cudaStreamSynchronize(P_->s);
-    if (e || !b) return e;
-    if ((e = cudaMemsetAsync(bar_.w, 0, sizeof(unsigned) * kGridBarWords, P_->s))) return e;
-    for (Sched* q : {&P_->schedA, &P_->schedAt, &P_->schedF, &P_->schedFt, &P_->schedQ})
-      if (q->cnt && (e = cudaMemsetAsync(q->cnt, 0, sizeof(int) * q->n_items, P_->s))) return e;
-    return cudaErrorTimeout;
-  }
-
   // One launch of the iteration's half-step on schedule q (0: A, the dual step;
   // 1: A^T, the primal step) with its own epilogue, on the engine's iterate
   // buffers: tuning runs before the iterate is initialised, so what these
@@ -1648,8 +1682,7 @@ class Engine final : public EngineBase {
   T *yavg_ = nullptr, *yanc_ = nullptr;
   T *Ds_ = nullptr, *fval_ = nullptr, *ftval_ = nullptr, *uvec_ = nullptr, *uvec2_ = nullptr;
   T *qv_ = nullptr, *qvec_ = nullptr, *qvec2_ = nullptr;  // general sparse Q
-  GridBar bar_{nullptr};     // barrier and chunk sums of power_rounds
-  double* csum_ = nullptr;
+  RoundState* rs_ = nullptr;  // power iteration by power_step
   int sms_ = 1;
   DevState* st_ = nullptr;
   HostStatus* hs_ = nullptr;

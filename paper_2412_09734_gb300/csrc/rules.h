@@ -10,14 +10,10 @@
 
 namespace mpax {
 
-// Whether round t of a power iteration whose state says `done` (the round that ended it, 0
-// while it runs) has nothing to do.  The launch that ends round t writes done = t while
-// other blocks of it still read the word, so both values must decide alike: warps of one
-// block that disagreed would leave the others alone at the block's barriers.
+// Whether launch t of a power iteration whose state says `done` (the launch that ended it, 0
+// while it runs) has nothing to do.  Launch t itself may write done = t while other blocks
+// of it still read the word, so both values must decide alike: warps of one block that
+// disagreed would leave the others alone at the block's barriers.
 MPAX_RULE bool power_round_over(int done, int t) { return done != 0 && done != t; }
-
-// Whether a barrier that waits for `phase` arrivals in all is open at `arrived`.  Both count
-// up modulo 2^32 (a launch of many million rounds passes it), never more than 2^31 apart.
-MPAX_RULE bool barrier_open(unsigned arrived, unsigned phase) { return (int)(arrived - phase) >= 0; }
 
 }  // namespace mpax

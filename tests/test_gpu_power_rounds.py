@@ -72,10 +72,10 @@ def test_norm_sum_over_very_many_items(C, rows):
 
 
 @pytest.mark.parametrize("case", list(CASES))
-def test_single_launch_runs_and_agrees_with_launched_rounds(C, case):
-    """A caller that names the kernel of the products gets the rounds as launches of their
-    own: the same norms to the 1e-9 of the oracle's, and more launches in all (four a round
-    and at least two rounds against one)."""
+def test_short_rounds_run_and_agree_with_the_general_kernels(C, case):
+    """A caller that names the kernel of the products gets the rounds of the general kernels:
+    the same norms to the 1e-9 of the oracle's, and more launches in all (four a round against
+    at most two and one at the end, in four rounds or more)."""
     from paper_2412_09734_gb300.problem import Problem
     d = CASES[case]()
     p = Problem.from_dict(d)

@@ -66,28 +66,6 @@ int main() {
         assert all(over[d, t] == 1 for d in range(1, t))
 
 
-def test_barrier_opens_with_its_last_arrival_past_the_counter_s_range_too(run_cpp):
-    """152 blocks arrive at barrier after barrier: closed until the last has arrived, open
-    from then on while the next barrier fills, on both sides of 2^32 arrivals."""
-    lines = run_cpp(r"""
-#include <cstdio>
-#include <initializer_list>
-#include "rules.h"
-int main() {
-  const unsigned blocks = 152;
-  for (unsigned start : {0u, 4294967000u, 4294967295u})
-    for (unsigned b = 1; b < 6; ++b)
-      for (int d = -(int)blocks; d <= (int)blocks; ++d) {
-        const unsigned phase = start + b * blocks;
-        std::printf("%d %d\n", d, (int)mpax::barrier_open(phase + (unsigned)d, phase));
-      }
-}
-""")
-    assert len(lines) > 4000
-    for d, is_open in (map(int, line.split()) for line in lines if line):
-        assert is_open == (d >= 0), d
-
-
 def test_scaled_value_from_float_pairs_is_the_fp64_product(run_cpp):
     """Bit for bit, for values and factors over the whole float range and near 1, and for
     zeros, infinities and NaN."""
