@@ -129,8 +129,10 @@ __global__ void __launch_bounds__(SgShape<BM, BN, TM, TN, BK, STAGES>::kThreads)
 }
 
 // Launch with the largest tile that still gives most SMs a CTA: large tiles reuse their
-// fragments most, but a tile's k chain takes about 28 ns per step whatever its size, so
-// idle SMs cost more.  Measured, microseconds of A~ V / A~^T V (128 x 128 tiles of the
+// fragments most, but idle SMs cost more.  At 1018 x 2050 x 100 a k step takes a CTA 28 ns with
+// 32 x 32 tiles (two warps), 31 with 64 x 32 (four) and 116 with 128 x 128 (eight): the few
+// warps' issue slots and four-byte copies, not the chain of an output, which a dependent FMA
+// lengthens by about 2 ns a step.  Measured, microseconds of A~ V / A~^T V (128 x 128 tiles of the
 // register-staged kernel before: first column):
 //   1018 x 2050 x 100    317 / 158    32 x 32: 57 / 35    64 x 32: 64 / 31    128 x 128: 238 / 113
 //   2036 x 4100 x 500    660 / 666    32 x 32: 356 / 352  64 x 32: 330 / 312  128 x 128: 441 / 431
