@@ -33,9 +33,9 @@ namespace mpax {
 // 40 ms).  FP32: one CTA of 1024 at 64 registers, or two of 512 where there are more
 // instances than such CTAs and they are small, at most kSmallCols columns on average and
 // kSmallVec rows and columns each: their slices of 32 rows leave many of 32 warps idle.
-// Measured, 1024 / 2 x 512 threads: 2,000 instances of 320 columns on average 13.2 / 8.6 ms,
-// 1,500 of 850 12.9 / 10.2, 1,000 of 1,200 12.3 / 10.5, 2,000 of 2,050 56 / 71; 100 of 620
-// 3.2 / 3.7.
+// Measured, 640 iterations, 1024 / 2 x 512 threads: 2,000 instances of 320 columns on average
+// 27.3 / 17.7 ms, 1,500 of 900 38.7 / 32.3, 1,000 of 1,200 34.9 / 31.1; in whole solves 2,000 of
+// 2,050 56 / 71 and 100 of 620 3.2 / 3.7.
 template <typename T>
 constexpr int kBatchThreads = sizeof(T) == 4 ? 1024 : 512;
 constexpr int kBatchSmallThreads = 512;
