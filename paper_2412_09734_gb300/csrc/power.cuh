@@ -2,10 +2,10 @@
 //
 // A round is two products, a reduction and a few scalars; as launches of the general kernels
 // it took two SpMVs, two small kernels and every eighth time a host round trip, and a problem
-// may need 50 to 450 rounds.  Here a product's launch first adds the partial sums that the
-// round before left and evaluates the stop rule, every CTA for itself, so a round is two
-// launches (one for a general Q); a problem of a few work items takes all its rounds in ONE
-// launch of one CTA.  Microseconds per round, general kernels -> here, FP64 and FP32:
+// may need 50 to 450 rounds.  Here every CTA of a round's first launch adds the partial sums
+// that the round before left, for the scale of v, and one CTA more evaluates the stop rule
+// meanwhile, so a round is two launches (one for a general Q); a problem of a few work items
+// takes all its rounds in ONE launch of one CTA.  Microseconds per round, general kernels -> here, FP64 and FP32:
 //   LP 200 x 400 (one CTA)      24.5 -> 12.4    23.3 -> 11.1
 //   LP 20,000 x 40,000          32.5 -> 22.3    25.5 -> 18.2
 //   LP 150,000 x 99,000         59.0 -> 38.9    36.6 -> 30.1
